@@ -57,7 +57,7 @@ SWEEP_TRAFFIC = {
     # 14,094,586,368 bytes read + 3,376,537,088 written
     "grid18m_k64": ("b2ee130f3957ab02", {"core_vertices": 20000}, 17471123456),
 }
-SWEEP_SOURCES = ("k_sweep_tma.cu", "iso_device.cuh", "schedule.cpp")
+SWEEP_SOURCES = ("k_tiles.cu", "tiles.cpp", "k_sweep_tma.cu", "sweep_device.cuh", "iso_device.cuh", "schedule.cpp")
 # sweep options that change the kernel's memory traffic, with their defaults
 # (0 = the library's automatic choice)
 TRAFFIC_OPTS = ("threads_per_vertex", "schedule_delay", "chunk_span", "solo_width", "fuse_width", "ctas_per_sm",
@@ -542,12 +542,16 @@ def main():
     achieved = alg / (sw / 1e3) / 1e9
     traffic = sweep_traffic(args.workload, opts)
     info = ws.sweep_info()
-    kern = f"k_sweep_tma<{K}>" if not info["core_levels"] else f"k_core + k_sweep_tma<{K}>"
+    # the sweep kernel that the options select (iso.h: sweep_kernel)
+    chunked = any(opts.get(key) for key in ("threads_per_vertex", "ctas_per_sm", "fuse_width", "sweep_kernel",
+                                            "schedule_delay", "solo_width", "chunk_span", "restrict_sweep",
+                                            "fused_emission"))
+    kern = ("k_core + " if info["core_levels"] else "") + (f"k_sweep_tma<{K}>" if chunked else f"k_tiles<{K}>")
     roof = {"bound": "hbm", "achieved": round(achieved, 1), "peak": peak, "unit": "GB/s",
             "frac": round(achieved / peak, 4), "traffic": traffic, "kernel": kern,
             "alg_bytes_per_launch": alg, "alg_bytes_design": alg_design,
             "traffic_over_alg": None if traffic is None else round(traffic / alg, 3),
-            "traffic_kernel": None if traffic is None else f"k_sweep_tma<{K}> (k_core's own bytes not counted)",
+            "traffic_kernel": None if traffic is None else f"{kern.split()[-1]} (k_core's own bytes not counted)",
             "peak_source": src, "sweep_ms": round(sw, 4), "lanes_per_launch": K}
     lat = sorted(pipelined["latency_ms"])
     line = {"metric": METRIC, "value": round(value, 2), "unit": "queries/s", "n_gpus": world, "steps": args.steps,

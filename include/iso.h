@@ -173,7 +173,11 @@ typedef struct {
     int32_t debug_barrier_extra;/* testing only: the sweep's barriers and dependency checks wait
                                    for this many extra arrivals or flags that never come, so the
                                    sweep times out */
-    int32_t sweep_kernel;       /* 0 = auto (TMA-staged arc blocks), 1 = TMA-staged, 2 = plain loads */
+    int32_t sweep_kernel;       /* 0 = auto: tiles swept out of shared memory, or the TMA-staged chunk
+                                   schedule where another option asks for it (threads_per_vertex,
+                                   ctas_per_sm, fuse_width, schedule_delay, solo_width, chunk_span,
+                                   debug_stage_*, restrict_sweep, fused_emission) or a vertex has too
+                                   many arcs for a tile; 1 = chunk schedule, 2 = plain loads */
     int32_t record_trace;       /* 1 = record the device time of every sweep step (iso_workspace_trace) */
     int32_t schedule_delay;     /* TMA-staged sweep: a chunk is scheduled at least this many positions
                                    after the chunks it depends on; 0 = auto (three times the CTA count) */
@@ -187,8 +191,8 @@ typedef struct {
     int32_t core_vertices;      /* TMA-staged sweep: the top level blocks of the hierarchy, as long as
                                    they hold at most this many vertices in total, are swept for each
                                    lane by one CTA with the lane's labels in shared memory (Section 5's
-                                   small top graph swept first); 0 = auto (the most that fit, 53,248),
-                                   -1 = never */
+                                   small top graph swept first); 0 = auto (the most that fit, 53,248;
+                                   20,000 above tiles), -1 = never */
     int32_t debug_stage_arcs;   /* testing only (TMA-staged sweep): stage at most this many arcs per
                                    chunk in shared memory (0 = the buffer size, 3,072); chunks with
                                    more read their arcs from global memory */
@@ -260,7 +264,7 @@ int iso_collect_range(iso_workspace* ws, uint32_t* out_bits, int64_t words_per_q
  * [0] upward search, [1] sweep, [2] emission, [3] sort + gather. */
 int iso_workspace_timings(const iso_workspace* ws, float* ms4);
 /* Per-level times of the last collected batch (workspaces created with
- * record_trace = 1 and the TMA-staged sweep).  Entry i < L: steps4[4i..4i+3] =
+ * record_trace = 1 and any sweep but the plain one).  Entry i < L: steps4[4i..4i+3] =
  * {0, i, i+1, 0} and ns[i] = device nanoseconds from the start of the sweep
  * until level block i was complete (blocks in sweep order, block 0 = top
  * level; below the leading levels the sweep interleaves levels, so these need
@@ -269,9 +273,12 @@ int iso_workspace_timings(const iso_workspace* ws, float* ms4);
  * the label rows).  Returns L+1 (at most cap entries are written) or -1 on
  * error. */
 int32_t iso_workspace_trace(const iso_workspace* ws, int32_t* steps4, int64_t* ns, int32_t cap);
-/* Shape of a workspace's sweep on its graph (TMA-staged sweep; zeros for the
- * plain one): how the level blocks are split between the phases and the chunk
- * schedule's extremes against the shared-memory staging limits. */
+/* Shape of a workspace's sweep on its graph (zeros for the plain one): how the
+ * level blocks are split between the phases and the chunk schedule's extremes
+ * against the shared-memory staging limits.  Tile sweep: core_levels =
+ * solo_levels = sync_levels, chunks are tiles, max_chunk_deps is the most label
+ * rows that a tile reads from outside, arc_cap and dep_cap bound a tile's arcs and
+ * rows. */
 typedef struct {
     int32_t levels;              /* level blocks L */
     int32_t core_levels;         /* blocks 0 .. core_levels-1: per-lane core */

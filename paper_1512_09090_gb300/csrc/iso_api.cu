@@ -2,8 +2,10 @@
 //
 // A batch of up to K lanes runs as one fixed launch sequence on the caller's
 // stream (optionally captured once into a CUDA graph and replayed):
-//   memset control block -> k_upward (one CTA per lane) -> k_sweep (persistent,
-//   cooperative) -> k_emit -> k_sort_gather [-> k_dist] -> copy summary to host.
+//   memset control block -> k_upward (one CTA per lane) -> k_core (the top of the
+//   hierarchy, one CTA per lane) -> k_tiles, or k_sweep_tma or k_sweep where options
+//   ask for them (persistent, cooperative) -> k_emit -> k_sort_gather [-> k_dist]
+//   -> copy summary to host.
 // Collecting waits for the summary, grows internal buffers and replays the
 // batch if an upward search or an emission list outgrew them, then copies the
 // lists (and labels) to the caller.  No step falls back to the CPU: without a
@@ -22,6 +24,7 @@
 #include "../../include/iso.h"
 #include "graph_view.h"
 #include "landmarks.h"
+#include "tiles.h"
 
 namespace {
 
@@ -70,6 +73,10 @@ bool is_device_ptr(const void* p) {
 }
 
 constexpr int kMaxLanes = 64;
+// Largest per-lane core above the tiles, by default: the core's blocks cost one SM
+// more the wider they get, a tier of tiles about 15 us.  Sweep step on 18M, 64
+// lanes: 2.64 ms with 10,000 and with 20,000 vertices, 2.68 with 35,000.
+constexpr int kTileCore = 20000;
 // default size limit of the top levels that CTA 0 sweeps alone in the TMA
 // sweep (four vertices per consumer warp)
 constexpr int kSoloWidth = 124;
@@ -90,6 +97,16 @@ int core_limit_of(const iso_query_opts& o, int n) {
     return std::min(lim, n);
 }
 
+// The sweep goes tile by tile (k_tiles) unless an option asks for one of the other
+// kernels or shapes the chunk schedule: the tiles were faster on every graph and
+// lane class measured (18M: 2.58 against 3.72 ms at 64 lanes, 0.89 against 1.27 at
+// one; 4M: 0.81 against 1.15 and 0.42 against 0.70).
+bool wants_tiles(const iso_query_opts& o) {
+    return o.sweep_kernel == 0 && o.threads_per_vertex == 0 && o.ctas_per_sm == 0 && o.fuse_width == 0 &&
+           o.schedule_delay == 0 && o.solo_width == 0 && o.chunk_span == 0 && o.debug_stage_arcs == 0 &&
+           o.debug_stage_deps == 0 && o.restrict_sweep == 0 && o.fused_emission == 0;
+}
+
 // Sweep kernel, threads per vertex, CTAs per SM and vertices per CTA batch that
 // options o select for K lanes.  Returns false if the combination is unsupported.
 bool sweep_shape(int K, const iso_query_opts& o, int* kernel, int* tpv, int* occ, int* vpb) {
@@ -108,6 +125,21 @@ bool sweep_shape(int K, const iso_query_opts& o, int* kernel, int* tpv, int* occ
 }
 
 }  // namespace
+
+// A tile plan on the device, shared by the workspaces with its lane class and core.
+struct TileDevice {
+    Allocator A;
+    cudaStream_t stream = nullptr;
+    int K = 0, core_n = 0, tiers = 0, count = 0, max_arcs = 0, max_ext = 0;
+    TileLimits lim{};
+    int32_t* off = nullptr;
+    uint2* dir = nullptr;
+    uint4* blob = nullptr;
+    int32_t* level_tier = nullptr;
+    ~TileDevice() {
+        for (void* p : {(void*)off, (void*)dir, (void*)blob, (void*)level_tier}) A.put(p, stream);
+    }
+};
 
 struct iso_graph {
     int device = 0;
@@ -146,12 +178,14 @@ struct iso_graph {
     std::vector<int32_t> h_level_off;
     // host copies for building sweep schedules
     std::vector<uint32_t> h_down_off;
-    std::vector<int32_t> h_down_src, h_bfs;
+    std::vector<int32_t> h_down_src, h_down_len, h_bfs;
     struct CachedSchedule {
         int vpb, narrow_width, sync_levels, delay, chunk_span;
         std::shared_ptr<SweepSchedule> s;
     };
     std::vector<CachedSchedule> schedules;
+    std::vector<std::shared_ptr<TileDevice>> plans;  // tile plans in use or used lately (kMaxPlans idle ones at most)
+    std::mutex plan_mu;
     std::mutex mu;
     iso_workspace* query_ws[7] = {};
     std::vector<void*> owned;
@@ -206,6 +240,8 @@ struct iso_workspace {
     int Q = 0;
     unsigned long long* upmask = nullptr;  // [n] TMA sweep: lanes with upward labels
     uint32_t* core_out = nullptr;  // [K * core_n] TMA sweep: the per-lane core's labels, lane-major
+    bool want_tiles = false;       // the options leave the sweep to the library
+    std::shared_ptr<TileDevice> tiles;  // tile sweep (null: chunk schedule or plain sweep)
     int vpb = 0;
     int2* pairs = nullptr;
     uint32_t* gtab = nullptr;
@@ -264,6 +300,59 @@ struct iso_workspace {
 
 namespace {
 
+constexpr size_t kMaxPlans = 6;  // one per lane class
+
+// Level blocks of the per-lane core: the longest run of top ones whose vertices fit `limit`.
+int core_levels_of(const iso_graph* g, int limit) {
+    int core = 0;
+    while (core < g->L && core < kCoreMaxLevels && g->h_level_off[core + 1] <= limit) ++core;
+    return core;
+}
+
+// The tile plan for K lanes below a core of core_n vertices (built once per
+// graph and kept while a workspace uses it), or null where there is none: a
+// vertex with too many sources, or no memory for it.
+std::shared_ptr<TileDevice> tile_plan(iso_graph* g, int K, int core_n) {
+    std::lock_guard<std::mutex> lock(g->plan_mu);
+    for (auto& t : g->plans)
+        if (t->K == K && t->core_n == core_n) return t;
+    auto t = std::make_shared<TileDevice>();
+    t->A = g->A;
+    t->stream = g->stream;
+    t->K = K;
+    t->core_n = core_n;
+    t->lim = iso_tile_limits(K);
+    try {
+        TilePlan plan;
+        if (iso_make_tiles(g->n, g->L, g->h_level_off.data(), g->h_down_off.data(), g->h_down_src.data(),
+                           g->h_down_len.data(), g->h_bfs.data(), core_n, t->lim, &plan) != 0)
+            return nullptr;
+        t->tiers = plan.tiers;
+        t->count = plan.tier_off.back();
+        t->max_arcs = plan.max_arcs;
+        t->max_ext = plan.max_ext;
+        auto put = [&](auto** dst, const auto& v) {
+            const size_t bytes = v.size() * sizeof(v[0]);
+            *(void**)dst = g->A.get(bytes, g->stream);
+            return *dst && (bytes == 0 || cudaMemcpyAsync(*dst, v.data(), bytes, cudaMemcpyHostToDevice, g->stream) ==
+                                              cudaSuccess);
+        };
+        if (!put(&t->off, plan.tier_off) || !put(&t->dir, plan.dir) || !put(&t->blob, plan.blob) ||
+            !put(&t->level_tier, plan.level_tier) || cudaStreamSynchronize(g->stream) != cudaSuccess) {
+            cudaStreamSynchronize(g->stream);  // no copy may outlive the host arrays
+            cudaGetLastError();
+            return nullptr;
+        }
+    } catch (const std::bad_alloc&) {
+        return nullptr;
+    }
+    for (size_t i = 0; i < g->plans.size() && g->plans.size() >= kMaxPlans;)
+        if (g->plans[i].use_count() == 1) g->plans.erase(g->plans.begin() + i);
+        else ++i;
+    g->plans.push_back(t);
+    return t;
+}
+
 int build_schedule(iso_workspace* ws) {
     iso_graph* g = ws->g;
     std::vector<int4> steps;
@@ -285,7 +374,18 @@ int build_schedule(iso_workspace* ws) {
     if (!ws->sched) { iso::set_error("workspace: device allocation failed"); return ISO_E_NOMEM; }
     ISO_CK(cudaMemcpyAsync(ws->sched, steps.data(), steps.size() * sizeof(int4), cudaMemcpyHostToDevice,
                            ws->stream));
-    if (ws->kernel == 1) {
+    if (ws->tiles) {
+        const TileDevice& t = *ws->tiles;
+        iso_sweep_info& in = ws->info;
+        in.levels = g->L;
+        in.core_levels = in.solo_levels = in.sync_levels = ws->core_levels;
+        in.core_vertices = ws->core_n;
+        in.chunks = t.count;
+        in.max_chunk_arcs = t.max_arcs;
+        in.max_chunk_deps = t.max_ext;
+        in.arc_cap = t.lim.blob_bytes / 8;
+        in.dep_cap = t.lim.rows;
+    } else if (ws->kernel == 1) {
         // TMA sweep: locality-ordered chunk schedule, cached on the graph
         const int delay = ws->sched_delay;
         // The leading levels sweep level by level before the schedule: those
@@ -293,8 +393,7 @@ int build_schedule(iso_workspace* ws) {
         // narrower than narrow_width in all CTAs with a grid barrier per level.
         // The per-lane core: the longest run of top level blocks whose vertices
         // fit core_limit (it replaces the CTA-0-alone levels).
-        int core = 0;
-        while (core < g->L && core < kCoreMaxLevels && g->h_level_off[core + 1] <= ws->core_limit) ++core;
+        const int core = core_levels_of(g, ws->core_limit);
         ws->core_levels = core;
         ws->core_n = g->h_level_off[core];
         int solo = core;
@@ -456,7 +555,12 @@ int enqueue(iso_workspace* ws, bool want_dist, bool capturing) {
     sw.ecap = ws->ecap;
     sw.sync_n = g->h_level_off[ws->sync_levels];
     if (ws->kernel == 1 && ws->core_levels > 0) ISO_CK(iso_launch_core(sw, K, s));
-    if (ws->kernel == 1) ISO_CK(iso_launch_sweep_tma(sw, K, ws->tpv, ws->grid, s));
+    if (ws->tiles) {
+        const TileDevice& t = *ws->tiles;
+        sw.tile_off = t.off; sw.tile_dir = t.dir; sw.tile_blob = t.blob; sw.level_tier = t.level_tier;
+        sw.tiers = t.tiers; sw.tile_lim = t.lim;
+        ISO_CK(iso_launch_tiles(sw, K, ws->grid, s));
+    } else if (ws->kernel == 1) ISO_CK(iso_launch_sweep_tma(sw, K, ws->tpv, ws->grid, s));
     else ISO_CK(iso_launch_sweep(sw, K, ws->tpv, ws->grid, s));
     ISO_CK(record(ws->ev[2], s, capturing));
     ISO_CK(record(ws->ev_swept, s, capturing));
@@ -570,7 +674,7 @@ extern "C" int iso_upload_graph(const iso_ch* ch, const iso_alloc* alloc, void* 
     const size_t n = (size_t)ch->n;
     std::vector<uint32_t> off32(n + 5);  // four spare entries keep 16-byte bulk copies in bounds
     std::vector<int2> arcs;
-    std::vector<int32_t> dsrc;
+    std::vector<int32_t> dsrc, dlen;
     int rc = ISO_OK;
     auto free_all = [&]() { for (void* p : g->owned) g->A.put(p, g->stream); g->owned.clear(); };
     // Emission entries for fused emission (Section 5): every input arc except
@@ -616,14 +720,16 @@ extern "C" int iso_upload_graph(const iso_ch* ch, const iso_alloc* alloc, void* 
         if (md > 0xFFFFFFF0u) { free_all(); iso::set_error("iso_upload_graph: too many downward arcs"); return ISO_E_INVAL; }
         arcs.resize(md + 2);  // two spare entries keep 16-byte loads in bounds
         dsrc.resize(md);
+        dlen.resize(md);
         size_t o = 0;
         for (size_t v = 0; v < n; ++v) {
             off32[v] = (uint32_t)o;
             for (int64_t a = ch->down_off[v]; a < ch->down_off[v + 1]; ++a, ++o) {
                 arcs[o] = make_int2(ch->down_src[a], ch->down_w[a]);
                 dsrc[o] = ch->down_src[a];
+                dlen[o] = ch->down_w[a];
             }
-            for (int32_t hi : dummy[v]) { arcs[o] = make_int2(hi, 0x7FFFFFFF); dsrc[o] = hi; ++o; }
+            for (int32_t hi : dummy[v]) { arcs[o] = make_int2(hi, 0x7FFFFFFF); dsrc[o] = hi; dlen[o++] = 0x7FFFFFFF; }
         }
         off32[n] = (uint32_t)o;
     } catch (const std::bad_alloc&) {
@@ -658,6 +764,7 @@ extern "C" int iso_upload_graph(const iso_ch* ch, const iso_alloc* alloc, void* 
     try {
         g->h_down_off = off32;
         g->h_down_src = std::move(dsrc);
+        g->h_down_len = std::move(dlen);
         g->h_bfs = ch->bfs;
     } catch (const std::bad_alloc&) {
         free_all();
@@ -709,6 +816,7 @@ extern "C" void iso_free_graph(iso_graph* g) {
     if (!g) return;
     cudaDeviceSynchronize();
     for (auto*& ws : g->query_ws) { iso_free_workspace(ws); ws = nullptr; }
+    g->plans.clear();
     for (void* p : g->owned) g->A.put(p, g->stream);
     delete g;
 }
@@ -743,6 +851,17 @@ extern "C" int iso_workspace_create(iso_graph* g, int32_t lanes, const iso_query
     ws->solo_width = o.solo_width < 0 ? 0 : (o.solo_width > 0 ? o.solo_width : kSoloWidth);
     ws->chunk_span = o.chunk_span;
     ws->core_limit = core_limit_of(o, g->n);
+    ws->want_tiles = wants_tiles(o);
+    if (ws->want_tiles) {
+        const int core = core_levels_of(g, o.core_vertices == 0 ? std::min(kTileCore, g->n) : ws->core_limit);
+        const int per = iso_tiles_occupancy(ws->K, iso_tile_limits(ws->K));
+        if (per > 0) ws->tiles = tile_plan(g, ws->K, g->h_level_off[core]);
+        if (ws->tiles) {
+            ws->core_levels = core;
+            ws->core_n = g->h_level_off[core];
+            ws->grid = g->num_sms * per;
+        }
+    }
     ws->stage_arc_cap = o.debug_stage_arcs;
     ws->stage_pred_cap = o.debug_stage_deps;
     ws->restrict_sweep = o.restrict_sweep != 0;
@@ -1089,7 +1208,9 @@ bool same_config(const iso_workspace* ws, const iso_query_opts& o) {
     const int per_sm = o.ctas_per_sm ? std::min<int>(o.ctas_per_sm, occ) : occ;
     const int fuse = o.fuse_width == 0 ? vpb : (o.fuse_width < 0 ? 0 : o.fuse_width);
     const long long timeout = o.barrier_timeout_ns ? o.barrier_timeout_ns : 2000000000LL;
-    return ws->kernel == kernel && ws->tpv == tpv && ws->grid == ws->g->num_sms * per_sm &&
+    const bool tiles = wants_tiles(o);  // (then the grid is the tile sweep's, the same for all such options)
+    return ws->kernel == kernel && ws->tpv == tpv && ws->want_tiles == tiles &&
+           (tiles || ws->grid == ws->g->num_sms * per_sm) &&
            ws->fuse_width == fuse && ws->use_graph == (o.use_cuda_graph != 0) && ws->timeout_ns == timeout &&
            ws->bar_extra == o.debug_barrier_extra && ws->record_trace == (o.record_trace != 0 && kernel == 1) &&
            ws->sched_delay == (o.schedule_delay > 0 ? o.schedule_delay : 3 * ws->g->num_sms * per_sm) &&

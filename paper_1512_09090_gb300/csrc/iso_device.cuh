@@ -15,6 +15,8 @@
 
 #include <atomic>
 
+#include "tiles.h"
+
 namespace isod {
 
 constexpr uint32_t kInf = 0x7FFFFFFFu;
@@ -113,6 +115,13 @@ struct SweepParams {
     int32_t* ebuf;             // [K * ecap]
     int ecap;
     int sync_n;                // vertices swept before the chunk schedule (core + leading levels)
+    // tile kernel: the plan (tiles.h), tiers in sweep order
+    const int32_t* tile_off;   // [tiers + 1] first tile of each tier
+    const uint2* tile_dir;     // per tile {record start / 16 bytes, record bytes}
+    const uint4* tile_blob;    // the records
+    const int32_t* level_tier; // [L] last tier of each level block (-1: core)
+    int tiers;
+    TileLimits tile_lim;
 };
 
 // Restricted sweep: which chunks are out of range for every lane of a batch,
@@ -213,6 +222,11 @@ cudaError_t iso_launch_sweep(const isod::SweepParams& p, int K, int tpv, int gri
 int iso_sweep_occupancy(int K, int tpv, int* block);
 bool iso_sweep_supported(int K, int tpv);
 cudaError_t iso_launch_sweep_tma(const isod::SweepParams& p, int K, int tpv, int grid, cudaStream_t s);
+// Tile sweep (k_tiles.cu): limits of a tile at K lanes, CTAs per SM, launch
+// (after iso_launch_core when p.core_levels > 0).
+TileLimits iso_tile_limits(int K);
+int iso_tiles_occupancy(int K, const TileLimits& lim);
+cudaError_t iso_launch_tiles(const isod::SweepParams& p, int K, int grid, cudaStream_t s);
 // Per-lane core (k_core.cu): K CTAs; runs before iso_launch_sweep_tma when p.core_levels > 0.
 cudaError_t iso_launch_core(const isod::SweepParams& p, int K, cudaStream_t s);
 int iso_sweep_tma_occupancy(int K, int tpv, int* block, int* vpb);

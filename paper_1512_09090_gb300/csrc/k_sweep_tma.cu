@@ -42,7 +42,7 @@
 // Every wait (mbarrier, dependency flag, grid barrier) is bounded: past the
 // limit the kernel records kStTimeout, stops issuing copies, waits (bounded)
 // for the copies it already issued, and returns.
-#include "iso_device.cuh"
+#include "sweep_device.cuh"
 
 namespace {
 
@@ -60,11 +60,6 @@ constexpr int kRounds = 2;               // vertices per thread group in a chunk
 // stage buffer, else one.
 template <int TPV>
 __host__ __device__ constexpr int rounds_of() { return kRounds * (kConsumers / TPV) + 5 <= kOffCap ? kRounds : 1; }
-
-template <int K> struct MaskOf { using T = uint8_t; };
-template <> struct MaskOf<16> { using T = uint16_t; };
-template <> struct MaskOf<32> { using T = uint32_t; };
-template <> struct MaskOf<64> { using T = unsigned long long; };
 
 struct Meta {
     int v0, v1;   // vertices [v0, v1)
@@ -86,64 +81,6 @@ struct Smem {
     int finished[kStages];  // consumer warps done with the chunk in each stage
     int ready_it[kStages];  // chunk (CTA-local index + 1) whose dependencies were seen complete
 };
-
-__device__ __forceinline__ uint32_t sa(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ void mbar_init(unsigned long long* b, uint32_t count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(sa(b)), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx(unsigned long long* b, uint32_t tx) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(sa(b)), "r"(tx) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(unsigned long long* b) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(sa(b)) : "memory");
-}
-__device__ __forceinline__ bool mbar_try_wait(unsigned long long* b, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(sa(b)), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-// Non-blocking probe of phase `parity` (try_wait may suspend the thread for a
-// while; a polling loop that also watches other things must not).
-__device__ __forceinline__ bool mbar_test_wait(unsigned long long* b, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(sa(b)), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-__device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes, unsigned long long* b) {
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                     sa(dst)),
-                 "l"(src), "r"(bytes), "r"(sa(b))
-                 : "memory");
-}
-
-// Bounded wait for phase `parity` of barrier b.  false = gave up (status set).
-__device__ bool mbar_wait(unsigned long long* b, uint32_t parity, const SweepParams& p) {
-    if (mbar_try_wait(b, parity)) return true;
-    const unsigned long long t0 = global_ns();
-    for (uint32_t it = 1;; ++it) {
-        if (mbar_try_wait(b, parity)) return true;
-        if ((it & 63) == 0) {
-            if (*(volatile int32_t*)p.status != kStOk) return false;
-            if (global_ns() - t0 > (unsigned long long)p.timeout_ns || it > (1u << 28)) {
-                atomicCAS(p.status, kStOk, kStTimeout);
-                return false;
-            }
-        }
-    }
-}
 
 template <int LPT> struct Row { uint32_t x[LPT]; };
 
@@ -209,8 +146,6 @@ __device__ __forceinline__ int lane_of(int sub, int i) {
     if constexpr (LPT >= 4) return 4 * (sub + TPV * (i / 4)) + (i & 3);
     else return sub * LPT + i;
 }
-
-__device__ __forceinline__ void fence_acq_rel_gpu() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
 
 // Polling load of a completion flag.  Flags are read relaxed, so that all of a
 // pass's loads are in flight at once; the reader fences (acquire) once after
@@ -431,43 +366,6 @@ __device__ __forceinline__ void finish_level(const SweepParams& p, const Smem& s
     }
 }
 
-// Label rows and in-range masks of the core vertices from k_core's lane-major
-// output (final, clamped labels): thread t of a warp takes vertex v0 + t,
-// reading lane i's label from row i of the lane-major array (coalesced over
-// the warp) and writing its own label row; bit i of the mask is set iff lane
-// i's label is not kInf.
-template <int K>
-__device__ void core_rows(const SweepParams& p, int warp, int lane) {
-    using MaskT = typename MaskOf<K>::T;
-    const int cn = p.core_n;
-    for (int v0 = ((int)blockIdx.x * (kThreads / 32) + warp) * 32; v0 < cn; v0 += (int)gridDim.x * kThreads) {
-        const int v = v0 + lane;
-        if (v >= cn) continue;
-        const uint32_t* src = p.core_out + v;
-        unsigned long long bits = 0;
-        if constexpr (K >= 4) {
-#pragma unroll 4
-            for (int i = 0; i < K; i += 4) {
-                uint4 x;
-                x.x = __ldcg(src + (size_t)i * cn);
-                x.y = __ldcg(src + (size_t)(i + 1) * cn);
-                x.z = __ldcg(src + (size_t)(i + 2) * cn);
-                x.w = __ldcg(src + (size_t)(i + 3) * cn);
-                bits |= (unsigned long long)(x.x != kInf) << i | (unsigned long long)(x.y != kInf) << (i + 1) |
-                        (unsigned long long)(x.z != kInf) << (i + 2) | (unsigned long long)(x.w != kInf) << (i + 3);
-                reinterpret_cast<uint4*>(p.d + (size_t)v * K)[i / 4] = x;
-            }
-        } else {
-            for (int i = 0; i < K; ++i) {
-                const uint32_t x = __ldcg(src + (size_t)i * cn);
-                bits |= (unsigned long long)(x != kInf) << i;
-                p.d[(size_t)v * K + i] = x;
-            }
-        }
-        static_cast<MaskT*>(p.mask)[v] = (MaskT)bits;
-    }
-}
-
 // Fused emission (Section 5: isochrone edges found by a second look at the
 // arcs of a vertex once its label is final).  Input arc e = (a, b) is checked
 // at its later-swept endpoint v against the other one, h, which is final
@@ -516,53 +414,6 @@ __device__ void emit_vertices(const SweepParams& p, int v_first, int v_stride, i
             }
         }
     }
-}
-
-// Grid-wide barrier of the whole CTA (the launch is cooperative, so every CTA
-// is resident): an arrival counter that the last arriver resets before it
-// advances a generation word the others poll.  (A barrier on one ever-growing
-// counter, one release-add to arrive and acquire-polling to wait, passed the
-// grid-synchronous levels about 70 us sooner on the 18M graph but left the
-// chunk phase that follows it 0.6 ms slower, with relaxed polling as well;
-// this one is kept.)  Bounded: gives up, recording kStTimeout, after the
-// timeout (bar_extra adds arrivals that never come, for the tests).  Returns
-// false, the same on every thread of the CTA, if the kernel has failed.
-__device__ bool grid_sync(const SweepParams& p) {
-    __shared__ int s_ok;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int ok = 1;
-        volatile int32_t* st = p.status;
-        volatile uint32_t* gen = p.bar + 1;
-        if (*st != kStOk) {
-            ok = 0;
-        } else {
-            const uint32_t g0 = *gen;
-            fence_acq_rel_gpu();
-            const uint32_t want = gridDim.x + (uint32_t)p.bar_extra;
-            if (atomicAdd(p.bar, 1u) + 1u == want) {
-                atomicExch(p.bar, 0u);
-                fence_acq_rel_gpu();
-                atomicAdd(p.bar + 1, 1u);
-            } else {
-                const unsigned long long t0 = global_ns();
-                for (uint32_t it = 0; *gen == g0; ++it) {
-                    if ((it & 15) == 15) {
-                        if (*st != kStOk) { ok = 0; break; }
-                        if (global_ns() - t0 > (unsigned long long)p.timeout_ns || it > (1u << 28)) {
-                            atomicCAS(p.status, kStOk, kStTimeout);
-                            ok = 0;
-                            break;
-                        }
-                    }
-                }
-            }
-            fence_acq_rel_gpu();
-        }
-        s_ok = ok;
-    }
-    __syncthreads();
-    return s_ok != 0;
 }
 
 // The chunk held in `stage`, by one consumer warp (its share of the vertices).
@@ -668,7 +519,7 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads) k_sweep_tma(SweepPa
     // labels of its vertices lane-major; they become label rows and masks here,
     // complete for every CTA after a grid barrier.
     if (p.core_levels > 0) {
-        core_rows<K>(p, warp, lane);
+        core_rows<K, kThreads>(p, tid);
         if (!grid_sync(p)) return;  // the same in every thread of the CTA
     }
     if (tid == 0) {

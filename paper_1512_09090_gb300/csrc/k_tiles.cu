@@ -1,0 +1,402 @@
+// PHAST scanning phase (Section 2) for K queries at once, pruned at tau, tile by
+// tile out of shared memory.
+//
+// Same computation as k_sweep_tma.cu: d[v,i] = min(up_i(v), min over downward
+// arcs (u,v) of d[u,i] + len(u,v)), 0x7FFFFFFF when that exceeds tau_i; uint32
+// sums never wrap (labels <= 0x7FFFFFFF, lengths <= 0x7FFFFFFE).
+//
+// The plan (tiles.cpp) cuts the vertices below the per-lane core into tiles of
+// several levels each.  A persistent CTA takes a tile at a time:
+//   - the tile's record (own vertices, arcs, rows it needs) comes by one bulk
+//     copy, started while the tile before it is swept;
+//   - the label rows of sources outside the tile are copied into shared memory
+//     (cp.async, 16 bytes a thread, all of them in flight at once);
+//   - the own vertices are swept phase by phase, a CTA barrier after each, a
+//     group of TPV threads per vertex with two 16-byte quads of lanes per thread;
+//     rows read inside the tile go to shared memory, rows read by other tiles
+//     to global memory, and every vertex's in-range mask to global memory.
+// Tiles of one tier are independent; a grid barrier separates the tiers (20 on
+// 18M vertices).  All waits are bounded (status word).
+//
+// Bound: latency.  A tile of 50 vertices takes a CTA about 5 us, of which the rows
+// from outside are a third and five phases the rest (a phase: a serial chain of
+// shared-memory reads per four arcs of its largest vertex).  The sweep step (with
+// k_core) on 18M vertices, one GB300: 64 lanes 2.58 ms (chunk schedule 3.72), 16
+// lanes 1.30 (2.03), one lane 0.89 (1.27).
+#include "sweep_device.cuh"
+
+namespace {
+
+// A thread's lanes of a row: LPT = 4 consecutive ones, or two quads, `sub` and
+// `sub + TPV` of the row's, so that neighbouring threads' 16-byte accesses are
+// neighbours.  (K = 32 and 16: two or four vertices share an access of eight
+// threads; every other one takes its quads in the opposite order, which spreads
+// them over the banks.)  Element i is lane lane_at(i).
+template <int LPT> struct Lanes { uint32_t x[LPT]; };
+
+__device__ __forceinline__ uint4 lds128(uint32_t a) {
+    uint4 v;
+    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a) : "memory");
+    return v;
+}
+__device__ __forceinline__ uint32_t lds32(uint32_t a) {
+    uint32_t v;
+    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
+    return v;
+}
+
+// Byte offsets of the thread's (first and second) quad in a row.
+template <int K, int TPV>
+struct Place {
+    static constexpr int LPT = K / TPV;
+    uint32_t o1, o2;
+    __device__ __forceinline__ Place(int sub, int lane) {
+        const bool flip = LPT == 8 && TPV < 8 && ((lane / TPV) & 1);
+        o1 = LPT == 1 ? 0u : 16u * (uint32_t)(sub + (flip ? TPV : 0));
+        o2 = K == 64 ? o1 + 128u : 16u * (uint32_t)(sub + (flip ? 0 : TPV));
+    }
+    __device__ __forceinline__ int lane_at(int i) const { return (int)((i < 4 ? o1 : o2) / 4) + (i & 3); }
+};
+
+template <int K, int TPV>
+__device__ __forceinline__ Lanes<K / TPV> lds_lanes(uint32_t row, const Place<K, TPV>& at) {
+    Lanes<K / TPV> r;
+    if constexpr (K / TPV == 1) {
+        r.x[0] = lds32(row);
+    } else {
+        const uint4 v = lds128(row + at.o1);
+        r.x[0] = v.x; r.x[1] = v.y; r.x[2] = v.z; r.x[3] = v.w;
+        if constexpr (K / TPV == 8) {
+            const uint4 u = lds128(row + at.o2);
+            r.x[4] = u.x; r.x[5] = u.y; r.x[6] = u.z; r.x[7] = u.w;
+        }
+    }
+    return r;
+}
+
+template <int K, int TPV>
+__device__ __forceinline__ void st_lanes(uint32_t* row, const Place<K, TPV>& at, const Lanes<K / TPV>& r) {
+    if constexpr (K / TPV == 1) {
+        *row = r.x[0];
+    } else {
+        *reinterpret_cast<uint4*>(row + at.o1 / 4) = make_uint4(r.x[0], r.x[1], r.x[2], r.x[3]);
+        if constexpr (K / TPV == 8)
+            *reinterpret_cast<uint4*>(row + at.o2 / 4) = make_uint4(r.x[4], r.x[5], r.x[6], r.x[7]);
+    }
+}
+
+__device__ __forceinline__ void cp_async16(uint32_t* dst, const uint32_t* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(sa(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+constexpr int kThreads = 128;
+constexpr int kCtasPerSm = 5;     // what the limits below leave room for
+
+constexpr int kUpRows = 16;       // rows for upward labels (more flagged vertices read theirs in place)
+constexpr int kInPlace = kUpRows + 1;
+
+// Dynamic shared memory: two record buffers, the label rows (the tile's, then
+// kUpRows more), a byte per own vertex (0: no upward label, 1 + i: in row i of
+// the latter, kInPlace: in its global row), 16-byte aligned each.
+struct TileSmem {
+    int rows_at, flags_at, bytes;
+};
+template <int K>
+__host__ __device__ inline TileSmem tile_smem(const TileLimits& lim) {
+    TileSmem s;
+    s.rows_at = 2 * lim.blob_bytes;
+    s.flags_at = s.rows_at + (((lim.rows + kUpRows) * K * 4 + 15) & ~15);
+    s.bytes = s.flags_at + ((lim.blob_bytes / 8 + 15) & ~15);  // (a vertex record has 8 bytes)
+    return s;
+}
+
+template <int K, int TPV>
+__global__ void __launch_bounds__(kThreads, kCtasPerSm) k_tiles(SweepParams p) {
+    constexpr int LPT = K / TPV;
+    static_assert(TPV == (int)sizeof(typename MaskOf<K>::T), "a thread writes one byte of the mask word");
+    extern __shared__ __align__(128) unsigned char smem[];
+    __shared__ unsigned long long full[2];
+    __shared__ int s_off[kTileMaxTiers + 1];
+    __shared__ int s_up, s_up_v[kUpRows];
+    const TileSmem lay = tile_smem<K>(p.tile_lim);
+    uint32_t* const rows = reinterpret_cast<uint32_t*>(smem + lay.rows_at);
+    uint8_t* const flags = smem + lay.flags_at;
+    const int tid = threadIdx.x;
+    const int lane = tid & 31;
+    const int sub = tid % TPV;
+    const Place<K, TPV> at(sub, lane);
+
+    if (p.trace && tid == 0 && blockIdx.x == 0 && p.core_levels == 0)
+        p.trace[0] = p.trace[p.L + 1] = (long long)global_ns();
+    if (tid == 0) {
+        mbar_init(&full[0], 1);
+        mbar_init(&full[1], 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    uint32_t tau[LPT];
+#pragma unroll
+    for (int i = 0; i < LPT; ++i) {
+        const int32_t t = p.tau[at.lane_at(i)];
+        tau[i] = t < 0 ? 0u : (uint32_t)t;
+    }
+    for (int i = tid; i <= p.tiers; i += kThreads) s_off[i] = __ldg(p.tile_off + i);
+    if (tid == 0) s_up = 0;
+    __syncthreads();
+
+    // tiles of this CTA: blockIdx.x, + gridDim.x, ... of every tier.  Each one's
+    // record is fetched while the one before it is swept, across tiers too (it
+    // holds graph data only).  Thread 0 also reads a tile's place one tile ahead.
+    int next_t = 0, next_q = (int)blockIdx.x - (int)gridDim.x;  // the tile to fetch next
+    uint2 next_at = make_uint2(0u, 0u);
+    auto advance = [&]() {
+        next_q += (int)gridDim.x;
+        while (next_t < p.tiers && next_q >= s_off[next_t + 1] - s_off[next_t]) {
+            ++next_t;
+            next_q = (int)blockIdx.x;
+        }
+        if (tid == 0 && next_t < p.tiers) next_at = __ldg(p.tile_dir + s_off[next_t] + next_q);
+    };
+    auto fetch = [&](int b) {  // (thread 0)
+        mbar_expect_tx(&full[b], next_at.y);
+        bulk_load(smem + (size_t)b * p.tile_lim.blob_bytes, p.tile_blob + next_at.x, next_at.y, &full[b]);
+    };
+    advance();
+    int done = 0;            // tiles swept
+    int cur_t = next_t;      // tier of tile `done`
+    bool in_flight = false;  // thread 0: the copy of its record is on its way
+    if (tid == 0 && next_t < p.tiers) { fetch(0); in_flight = true; }
+    advance();
+
+    // labels of the per-lane core as rows and masks, complete after the first barrier
+    bool ok = true;
+    if (p.core_levels > 0) {
+        core_rows<K, kThreads>(p, tid);
+        if (p.tiers > 0 || p.bar_extra > 0) ok = grid_sync(p);
+    }
+    for (int t = 0; ok && t < p.tiers; ++t) {
+        while (cur_t == t) {
+            const int b = done & 1;
+            // its record is here; every thread of the CTA goes on or none
+            if (!__syncthreads_and(mbar_wait(&full[b], (uint32_t)(done >> 1) & 1u, p))) { ok = false; break; }
+            ++done;
+            in_flight = false;
+            const uint32_t* rec = reinterpret_cast<const uint32_t*>(smem + (size_t)b * p.tile_lim.blob_bytes);
+            const int n_ext = (int)rec[0], n_own = (int)rec[1], phases = (int)rec[2];
+            const uint2* vert = reinterpret_cast<const uint2*>(rec + rec[3]);
+            const uint2* arcs = reinterpret_cast<const uint2*>(rec + rec[4]);
+            const uint32_t* ext = rec + kTileHeader + phases;
+            // rows from outside (final: written before the last grid barrier)
+            if constexpr (K >= 4) {
+                for (int i = tid; i < n_ext * (K / 4); i += kThreads)
+                    cp_async16(rows + 4 * i, p.d + (size_t)ext[i / (K / 4)] * K + 4 * (i % (K / 4)));
+            } else {
+                for (int i = tid; i < n_ext; i += kThreads) rows[i] = __ldcg(p.d + ext[i]);
+            }
+            // the next tile's record
+            if (tid == 0 && next_t < p.tiers) { fetch(b ^ 1); in_flight = true; }
+            cur_t = next_t;
+            advance();
+            // upward labels of own vertices: a row each, kInf in the lanes whose search did not get there
+            bool up = false;
+            for (int i = tid; i < n_own; i += kThreads) {
+                const int v = (int)(vert[i].x & ~kTileStore);
+                int f = __ldcg(p.upflag + v);
+                if (f) {
+                    up = true;
+                    f = min(atomicAdd(&s_up, 1) + 1, kInPlace);
+                    if (f < kInPlace) s_up_v[f - 1] = v;
+                }
+                flags[i] = (uint8_t)f;
+            }
+            if constexpr (K >= 4) cp_async_wait();
+            up = __syncthreads_or(up);
+            if (up) {
+                constexpr int Q = K >= 4 ? K / 4 : 1;  // pieces of a row: four lanes, or the only one
+                for (int i = tid; i < min(s_up, kUpRows) * Q; i += kThreads) {
+                    const int v = s_up_v[i / Q], l = 4 * (i % Q);
+                    const unsigned long long um = __ldcg(p.upmask + v) >> l;
+                    uint32_t* const dst = rows + (p.tile_lim.rows + i / Q) * K + l;
+                    const uint32_t* const src = p.d + (size_t)v * K + l;
+                    if constexpr (K >= 4) {
+                        uint4 x = __ldcg(reinterpret_cast<const uint4*>(src));
+                        x.x = um & 1ull ? x.x : kInf;
+                        x.y = um & 2ull ? x.y : kInf;
+                        x.z = um & 4ull ? x.z : kInf;
+                        x.w = um & 8ull ? x.w : kInf;
+                        *reinterpret_cast<uint4*>(dst) = x;
+                    } else {
+                        const uint32_t x = __ldcg(src);
+                        *dst = um & 1ull ? x : kInf;
+                    }
+                }
+                __syncthreads();
+            }
+            // phases: the next one's vertex record is read before the barrier that ends
+            // the phase in front of it
+            const uint32_t rows_a = sa(rows), arcs_a = sa(arcs);
+            int hi = (int)rec[kTileHeader];
+            int j = tid / TPV;  // (at most kThreads / TPV vertices a phase)
+            uint2 me = vert[min(j, n_own)];
+            uint32_t e = vert[min(j + 1, n_own)].y;
+            for (int ph = 0; ph < phases; ++ph) {
+                const bool valid = j < hi;
+                const int v = (int)(me.x & ~kTileStore);
+                Lanes<LPT> acc;
+#pragma unroll
+                for (int i = 0; i < LPT; ++i) acc.x[i] = kInf;
+                // Labels above tau need no clamp here: they only ever give labels above
+                // tau, and acc stays <= kInf, so that sums cannot wrap.
+                const uint32_t end = valid ? arcs_a + 8u * (e & 0xFFFFu) : 0u;
+#pragma unroll 1
+                for (uint32_t a = arcs_a + 8u * (me.y & 0xFFFFu); a < end; a += 32u) {
+                    const uint4 q0 = lds128(a), q1 = lds128(a + 16u);
+                    const Lanes<LPT> r0 = lds_lanes<K, TPV>(rows_a + q0.x * (K * 4), at);
+                    const Lanes<LPT> r1 = lds_lanes<K, TPV>(rows_a + q0.z * (K * 4), at);
+                    const Lanes<LPT> r2 = lds_lanes<K, TPV>(rows_a + q1.x * (K * 4), at);
+                    const Lanes<LPT> r3 = lds_lanes<K, TPV>(rows_a + q1.z * (K * 4), at);
+#pragma unroll
+                    for (int i = 0; i < LPT; ++i) acc.x[i] = __viaddmin_u32(r0.x[i], q0.y, acc.x[i]);
+#pragma unroll
+                    for (int i = 0; i < LPT; ++i) acc.x[i] = __viaddmin_u32(r1.x[i], q0.w, acc.x[i]);
+#pragma unroll
+                    for (int i = 0; i < LPT; ++i) acc.x[i] = __viaddmin_u32(r2.x[i], q1.y, acc.x[i]);
+#pragma unroll
+                    for (int i = 0; i < LPT; ++i) acc.x[i] = __viaddmin_u32(r3.x[i], q1.w, acc.x[i]);
+                }
+                const int f = up && valid ? flags[j] : 0;
+                if (f == kInPlace) {  // only the lanes marked in upmask hold this batch's values
+                    const unsigned long long um = __ldcg(p.upmask + v);
+#pragma unroll
+                    for (int i = 0; i < LPT; ++i) {
+                        const int l = at.lane_at(i);
+                        if ((um >> l) & 1ull) acc.x[i] = min(acc.x[i], __ldcg(p.d + (size_t)v * K + l));
+                    }
+                } else if (f) {
+                    const Lanes<LPT> r = lds_lanes<K, TPV>(rows_a + (uint32_t)(p.tile_lim.rows + f - 1) * (K * 4), at);
+#pragma unroll
+                    for (int i = 0; i < LPT; ++i) acc.x[i] = min(acc.x[i], r.x[i]);
+                }
+                const uint32_t slot = me.y >> 16;
+                if (valid && slot != kTileNoRow) st_lanes<K, TPV>(rows + slot * K, at, acc);
+                // out-of-range bits: the sign of tau - label (both below 2^31), last element first
+                uint32_t bits = 0;
+#pragma unroll
+                for (int i = LPT - 1; i >= 0; --i) bits = __funnelshift_l(tau[i] - acc.x[i], bits, 1);
+                if (valid && ((me.x & kTileStore) || p.write_all)) {
+                    if (p.write_all) {  // distances are returned: out-of-range labels as kInf
+#pragma unroll
+                        for (int i = 0; i < LPT; ++i)
+                            if (acc.x[i] > tau[i]) acc.x[i] = kInf;
+                    }
+                    st_lanes<K, TPV>(p.d + (size_t)v * K, at, acc);
+                }
+                // one byte of the mask word per thread: with two quads, a thread and its
+                // neighbour swap a nibble each, the even one gets the lower quads' byte
+                bits = ~bits;
+                int byte = sub;
+                if constexpr (LPT == 8) {
+                    if (at.o1 > at.o2) bits = (bits >> 4 & 0xFu) | bits << 4;  // lower quad first
+                }
+                if constexpr (LPT == 8 && TPV > 1) {
+                    const uint32_t other = __shfl_xor_sync(0xffffffffu, bits, 1);
+                    bits = sub & 1 ? (other >> 4 & 0xFu) | (bits & 0xF0u) : (bits & 0xFu) | (other & 0xFu) << 4;
+                    byte = sub / 2 + (sub & 1) * (TPV / 2);
+                }
+                if (valid) static_cast<uint8_t*>(p.mask)[(size_t)v * TPV + byte] = (uint8_t)(bits & ((1u << LPT) - 1u));
+                if (ph + 1 < phases) {
+                    j = hi + tid / TPV;
+                    hi = (int)rec[kTileHeader + ph + 1];
+                    me = vert[min(j, n_own)];
+                    e = vert[min(j + 1, n_own)].y;
+                }
+                __syncthreads();
+            }
+            if (up) {  // the upward labels are used up
+                for (int i = tid; i < n_own; i += kThreads)
+                    if (flags[i]) {
+                        const int v = (int)(vert[i].x & ~kTileStore);
+                        p.upflag[v] = 0;
+                        p.upmask[v] = 0ull;
+                    }
+                if (tid == 0) s_up = 0;
+            }
+        }
+        if (ok && (t + 1 < p.tiers || p.bar_extra > 0)) ok = grid_sync(p);
+        if (ok && p.trace)
+            for (int j = tid; j < p.L; j += kThreads)
+                if (p.level_tier[j] == t) atomicMax((unsigned long long*)p.trace + 1 + j, global_ns());
+    }
+    // a record copy still on its way lands before the CTA exits
+    if (tid == 0 && in_flight) mbar_wait(&full[done & 1], (uint32_t)(done >> 1) & 1u, p);
+}
+
+constexpr int kMaxSmem = 224 * 1024;  // dynamic shared memory a CTA may ask for (static arrays come on top)
+
+template <int K, int TPV>
+int occupancy(const TileLimits& lim) {
+    static std::atomic<unsigned long long> attr{0};
+    const int bytes = tile_smem<K>(lim).bytes;
+    int blocks = 0;
+    if (iso_smem_attr_once(k_tiles<K, TPV>, kMaxSmem, attr) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, k_tiles<K, TPV>, kThreads, bytes) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
+    return blocks;
+}
+
+template <int K, int TPV>
+cudaError_t launch(const SweepParams& p, int grid, cudaStream_t s) {
+    static std::atomic<unsigned long long> attr{0};
+    if (cudaError_t e = iso_smem_attr_once(k_tiles<K, TPV>, kMaxSmem, attr)) return e;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = (size_t)tile_smem<K>(p.tile_lim).bytes;
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeCooperative;
+    at[0].val.cooperative = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k_tiles<K, TPV>, p);
+}
+
+#define ISO_TILE_CASES(X) X(1, 1) X(4, 1) X(8, 1) X(16, 2) X(32, 4) X(64, 8)
+
+}  // namespace
+
+TileLimits iso_tile_limits(int K) {
+    // Five CTAs per SM (about 43 KB each): a tile costs mostly latency (rows from
+    // outside 1.4 us, 0.5 us a phase), so tiles in flight count for more than large
+    // tiles.  18M vertices, 64 lanes, ms of the whole sweep step: rows 100 (5 CTAs)
+    // 2.58, 120 2.61, 156 (4 CTAs) 2.71; comp 16 2.58, 12 2.58, 8 2.64.  16 lanes:
+    // rows 300 1.30, 220 1.41, 400 1.32; comp 16 1.30, 8 1.33, 32 1.33.  One lane:
+    // 1,500 rows and 16 KB 0.89 (comp 32; 16: 0.95), 1,000 and 10 KB 0.93.
+    TileLimits l{};
+    switch (K) {
+        case 64: l.rows = 100; l.blob_bytes = 6144; l.comp = 16; break;
+        case 32: l.rows = 200; l.blob_bytes = 8192; l.comp = 16; break;
+        case 16: l.rows = 300; l.blob_bytes = 10240; l.comp = 16; break;
+        case 8: l.rows = 600; l.blob_bytes = 12288; l.comp = 24; break;
+        case 4: l.rows = 1000; l.blob_bytes = 14336; l.comp = 32; break;
+        default: l.rows = 1500; l.blob_bytes = 16384; l.comp = 32; break;
+    }
+    l.width = kThreads / (K >= 8 ? K / 8 : 1);
+    return l;
+}
+
+int iso_tiles_occupancy(int K, const TileLimits& lim) {
+#define X(k, t) if (K == k) return occupancy<k, t>(lim);
+    ISO_TILE_CASES(X)
+#undef X
+    return 0;
+}
+
+cudaError_t iso_launch_tiles(const isod::SweepParams& p, int K, int grid, cudaStream_t s) {
+#define X(k, t) if (K == k) return launch<k, t>(p, grid, s);
+    ISO_TILE_CASES(X)
+#undef X
+    return cudaErrorInvalidValue;
+}
