@@ -172,7 +172,6 @@ struct iso_graph {
     uint32_t* lm_fwd = nullptr;
     uint32_t* lm_bwd = nullptr;
     std::atomic<int> restricted_ws{0};  // live workspaces with restricted sweeps (they use lm_*)
-    int32_t* perm = nullptr;
     int32_t* pos = nullptr;
     int32_t* level_off = nullptr;
     std::vector<int32_t> h_level_off;
@@ -586,7 +585,7 @@ int enqueue(iso_workspace* ws, bool want_dist, bool capturing) {
     ISO_CK(iso_launch_sort_gather(ga, K, s));
     if (want_dist) {
         DistParams dp{};
-        dp.d = ws->d; dp.perm = g->perm; dp.out = ws->dist; dp.n = g->n; dp.k = K; dp.K = K;
+        dp.d = ws->d; dp.pos = g->pos; dp.out = ws->dist; dp.n = g->n; dp.k = K; dp.K = K;
         ISO_CK(iso_launch_dist(dp, s));
     }
     ISO_CK(record(ws->ev[4], s, capturing));
@@ -800,7 +799,7 @@ extern "C" int iso_upload_graph(const iso_ch* ch, const iso_alloc* alloc, void* 
         (rc = g->upload(&g->orig_head, head.data(), head.size())) ||
         (rc = g->upload(&g->orig_id, aid.data(), aid.size())) ||
         (rc = g->upload(&g->emit_tail, tail.data(), n)) ||
-        (rc = g->upload(&g->perm, ch->perm.data(), n)) || (rc = g->upload(&g->pos, ch->pos.data(), n)) ||
+        (rc = g->upload(&g->pos, ch->pos.data(), n)) ||
         (rc = g->upload(&g->level_off, ch->level_off.data(), ch->level_off.size()))) {
         free_all(); return rc;
     }

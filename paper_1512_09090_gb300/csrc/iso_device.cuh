@@ -173,7 +173,7 @@ struct RangeParams {
 
 struct DistParams {
     const uint32_t* d;
-    const int32_t* perm;
+    const int32_t* pos;        // [n] original id -> sweep position
     int32_t* out;              // [k * n], query-major, original vertex order
     int n, k, K;
 };

