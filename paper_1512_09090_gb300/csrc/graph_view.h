@@ -12,9 +12,9 @@ struct iso_graph_view {
     int n, L, tau_max, num_sms;
     int device;  // CUDA device the graph was uploaded to
     int64_t m;
-    const uint32_t *down_off, *up_off, *orig_off;
-    const int2 *down_arc, *up_arc;
-    const int32_t *orig_head, *orig_id, *pos, *level_off, *emit_tail;
+    const uint32_t *down_off, *up_off, *pair_off;
+    const int2 *down_arc, *up_arc, *pair_ids;
+    const int32_t *pair_head, *pos, *level_off, *pair_owner;
     const int32_t* h_level_off;
 };
 

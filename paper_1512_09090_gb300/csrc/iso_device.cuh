@@ -140,10 +140,10 @@ struct SkipParams {
 };
 
 struct EmitParams {
-    const uint32_t* orig_off;  // [n+1] input arcs grouped by tail, by emission index
-    const int32_t* orig_head;  // sweep positions
-    const int32_t* orig_id;
-    const int32_t* tail_of;    // [n] sweep position of the tail at each emission index
+    const uint32_t* off;       // [n+1] vertex pairs by owner, owners by BFS rank (emit_pairs.h)
+    const int32_t* head;       // sweep position of each pair's other endpoint
+    const int2* ids;           // its arc ids {id, second id or -1}
+    const int32_t* owner;      // [n] sweep position of each owner
     const int32_t* status;     // batch status: emission is skipped once it is not kStOk
     const void* mask;
     int32_t* ecnt;             // [K]

@@ -190,8 +190,8 @@ extern "C" int iso_query_noalloc(iso_graph* g, int32_t k, const int32_t* sources
         return fail_enqueued(ISO_E_CUDA, "sweep launch", e, stream);
 
     EmitParams em{};
-    em.orig_off = gv.orig_off; em.orig_head = gv.orig_head; em.orig_id = gv.orig_id; em.mask = sw.mask;
-    em.tail_of = gv.emit_tail;
+    em.off = gv.pair_off; em.head = gv.pair_head; em.ids = gv.pair_ids; em.mask = sw.mask;
+    em.owner = gv.pair_owner;
     em.status = ctl;
     em.ecnt = ctl + 8; em.ebuf = (int32_t*)(base + kOffEbuf); em.n = gv.n; em.ecap = kMaxArcs;
     if ((e = iso_launch_emit(em, kLanes, gv.num_sms * 8, stream)) != cudaSuccess)

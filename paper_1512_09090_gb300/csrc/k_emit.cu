@@ -1,11 +1,9 @@
-// Isochrone edge emission (Section 3): arc (u,v) of the input graph is an
-// isochrone edge for lane i iff exactly one of u, v is in range, i.e. iff bit i
-// of mask[u] XOR mask[v] is set.  Arcs are visited grouped by tail, tails in
-// BFS order of the input graph: neighbouring warps then read the masks of
-// neighbouring vertices, which sit in a few short stretches of each level's
-// part of the mask array and stay in L2, instead of scattered sectors.  Per lane, ids are appended with one
-// atomicAdd per warp: __ballot_sync gives the warp's members for that lane and
-// __popc of the lower lanes gives each member's slot.
+// Isochrone edge emission (Section 3): an arc between u and h is an isochrone
+// edge for lane i iff exactly one of them is in range, i.e. iff bit i of mask[u]
+// XOR mask[h] is set.  Vertex pairs (emit_pairs.cpp: both arcs of a two-way road at
+// once) are visited in BFS order of their owners.  A CTA collects the edges it
+// finds in shared memory and takes room in the lists with one atomicAdd per query
+// for about a thousand of them.
 //
 // Then k_sort_gather sorts each lane's ids ascending (bucket sort in shared
 // memory, four CTAs per lane) and writes them to the contiguous output at the
@@ -22,41 +20,62 @@ template <> struct MaskOf<32> { using T = uint32_t; };
 template <> struct MaskOf<64> { using T = unsigned long long; };
 
 constexpr int kEmitThreads = 256;
-constexpr int kEmitBatch = 4;     // rounds of 32 arcs whose loads a warp has in flight together
+constexpr int kEmitBatch = 2;     // rounds of 32 pairs whose loads a warp has in flight together
+constexpr int kEmitBuffer = 2048; // edges a CTA collects before it takes room in the lists
 constexpr int kSortThreads = 1024;
 constexpr int kSortSmem = 16384;  // ids bucketed in shared memory (64 KB): two sorting CTAs fit an SM
 
-__device__ __forceinline__ unsigned long long warp_or(unsigned long long x) {
-    const unsigned lo = __reduce_or_sync(0xffffffffu, (unsigned)x);
-    const unsigned hi = __reduce_or_sync(0xffffffffu, (unsigned)(x >> 32));
-    return ((unsigned long long)hi << 32) | lo;
-}
-
+// Bound by latency: two dependent loads per pair (head, then its mask: 8 bytes
+// anywhere in a few stretches of the mask array).  Two rounds of 32 pairs in flight
+// per warp and all the warps an SM holds (64); the appends must not wait for a
+// counter each: one atomicAdd per warp, query and round (half a million of them on
+// 64 counters in two cache lines) kept the kernel at 0.32 ms however many warps it
+// had.  18M vertices, 64 queries (1.2M edges): 0.52 ms arc by arc with those
+// atomics, now 0.23 (0.35 GB to move); one query 0.34, now 0.16.
 template <int K>
 __global__ void __launch_bounds__(kEmitThreads) k_emit(EmitParams p) {
     using MaskT = typename MaskOf<K>::T;
     // bits of lanes that exist: a mask word holds at least 8 bits, and after a
     // failed sweep it may hold anything
     constexpr unsigned long long kLanes = K >= 64 ? ~0ull : ((1ull << K) - 1ull);
+    __shared__ int s_id[kEmitBuffer];       // edges found: arc id ...
+    __shared__ uint32_t s_to[kEmitBuffer];  // ... and query << 24 | place among the query's
+    __shared__ int s_n, s_cnt[K], s_base[K];
     // a failed batch (bad input, upward overflow, timeout) is reported by the
     // host; its masks may be stale, so nothing is emitted
     if (*(volatile const int32_t*)p.status != kStOk) return;
     const MaskT* mask = static_cast<const MaskT*>(p.mask);
     const unsigned lane = threadIdx.x & 31;
-    const unsigned lt = (1u << lane) - 1u;
-    const int warps = (int)(gridDim.x * blockDim.x) >> 5;
-    // a warp takes 32 consecutive tails (emission indices); their arcs are one
-    // contiguous range
-    for (int w = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); w * 32 < p.n; w += warps) {
-        const int u0 = w * 32;
+    for (int i = threadIdx.x; i < K; i += kEmitThreads) s_cnt[i] = 0;
+    if (threadIdx.x == 0) s_n = 0;
+    __syncthreads();
+    auto flush = [&]() {  // (the whole CTA)
+        for (int i = threadIdx.x; i < K; i += kEmitThreads)
+            s_base[i] = s_cnt[i] ? atomicAdd(p.ecnt + i, s_cnt[i]) : 0;
+        __syncthreads();
+        const int n = min(s_n, kEmitBuffer);
+        for (int e = threadIdx.x; e < n; e += kEmitThreads) {
+            if (s_to[e] == 0xFFFFFFFFu) continue;  // the buffer ended inside a pair
+            const int i = (int)(s_to[e] >> 24), q = s_base[i] + (int)(s_to[e] & 0xFFFFFFu);
+            if (q < p.ecap) p.ebuf[(size_t)i * p.ecap + q] = s_id[e];
+        }
+        __syncthreads();
+        for (int i = threadIdx.x; i < K; i += kEmitThreads) s_cnt[i] = 0;
+        if (threadIdx.x == 0) s_n = 0;
+        __syncthreads();
+    };
+    // a CTA takes kEmitThreads consecutive owners at a time, a warp 32 of them; a
+    // warp's pairs are one contiguous range
+    for (int64_t c0 = (int64_t)blockIdx.x * kEmitThreads; c0 < p.n; c0 += (int64_t)gridDim.x * kEmitThreads) {
+        const int u0 = (int)min(c0 + (threadIdx.x & ~31u), (int64_t)p.n);
         const int u = min(u0 + (int)lane, p.n);
-        const uint32_t my_off = __ldg(p.orig_off + u);           // start of tail u0+lane's arcs
+        const uint32_t my_off = __ldg(p.off + u);           // start of owner u0+lane's pairs
         const uint32_t a0 = __shfl_sync(0xffffffffu, my_off, 0);
-        const uint32_t a1 = __ldg(p.orig_off + min(u0 + 32, p.n));
-        const unsigned long long mu_lane = u < p.n ? (unsigned long long)mask[__ldg(p.tail_of + u)] : 0ull;
-        // kEmitBatch rounds of 32 arcs at a time: all their heads, then all the
-        // heads' masks are in flight together (two dependent round trips for up
-        // to 32 * kEmitBatch arcs instead of two per 32)
+        const uint32_t a1 = __ldg(p.off + min(u0 + 32, p.n));
+        const unsigned long long mu_lane =
+            u < p.n ? (unsigned long long)mask[__ldg(p.owner + u)] : 0ull;
+        // kEmitBatch rounds of 32 pairs at a time: all their heads, then all the
+        // heads' masks are in flight together
         for (uint32_t base0 = a0; base0 < a1; base0 += 32 * kEmitBatch) {
             unsigned long long mh[kEmitBatch];
             {
@@ -64,48 +83,52 @@ __global__ void __launch_bounds__(kEmitThreads) k_emit(EmitParams p) {
 #pragma unroll
                 for (int r = 0; r < kEmitBatch; ++r) {
                     const uint32_t a = base0 + 32 * r + lane;
-                    hd[r] = a < a1 ? __ldg(p.orig_head + a) : -1;
+                    hd[r] = a < a1 ? __ldg(p.head + a) : -1;
                 }
 #pragma unroll
                 for (int r = 0; r < kEmitBatch; ++r) mh[r] = hd[r] >= 0 ? (unsigned long long)mask[hd[r]] : 0ull;
             }
 #pragma unroll
             for (int r = 0; r < kEmitBatch; ++r) {
-            const uint32_t base = base0 + 32 * r;
-            if (base >= a1) break;  // warp-uniform
-            const uint32_t a = base + lane;
-            unsigned long long x = 0;
-            int id = 0;
-            // tail of arc a: the last lane t whose first arc is <= a
-            int lo = 0;
+                const uint32_t base = base0 + 32 * r;
+                if (base >= a1) break;  // warp-uniform
+                const uint32_t a = base + lane;
+                // owner of pair a: the last lane t whose first pair is <= a
+                int lo = 0;
 #pragma unroll
-            for (int step = 16; step > 0; step >>= 1) {
-                const uint32_t o = __shfl_sync(0xffffffffu, my_off, lo + step);
-                if (lo + step < 32 && o <= a) lo += step;
-            }
-            const unsigned long long mu = __shfl_sync(0xffffffffu, mu_lane, lo);
-            if (a < a1) {
-                x = (mu ^ mh[r]) & kLanes;
-                if (x) id = __ldg(p.orig_id + a);
-            }
-            if (!__any_sync(0xffffffffu, x != 0)) continue;
-            unsigned long long todo = warp_or(x);
-            while (todo) {
-                const int i = __ffsll((long long)todo) - 1;
-                todo &= todo - 1;
-                const unsigned b = __ballot_sync(0xffffffffu, (x >> i) & 1ull);
-                const int leader = __ffs(b) - 1;
-                int at = 0;
-                if ((int)lane == leader) at = atomicAdd(p.ecnt + i, __popc(b));
-                at = __shfl_sync(0xffffffffu, at, leader);
-                if ((x >> i) & 1ull) {
-                    const int q = at + __popc(b & lt);
-                    if (q < p.ecap) p.ebuf[(size_t)i * p.ecap + q] = id;
+                for (int step = 16; step > 0; step >>= 1) {
+                    const uint32_t o = __shfl_sync(0xffffffffu, my_off, lo + step);
+                    if (lo + step < 32 && o <= a) lo += step;
+                }
+                const unsigned long long mu = __shfl_sync(0xffffffffu, mu_lane, lo);
+                unsigned long long x = a < a1 ? (mu ^ mh[r]) & kLanes : 0ull;
+                if (x == 0) continue;
+                const int2 id = __ldg(p.ids + a);
+                const int each = id.y >= 0 ? 2 : 1;
+                for (int slot = atomicAdd(&s_n, each * __popcll(x)); x; x &= x - 1, slot += each) {
+                    const int i = __ffsll((long long)x) - 1;
+                    if (slot + each <= kEmitBuffer) {
+                        const uint32_t to = (uint32_t)i << 24 | (uint32_t)atomicAdd(&s_cnt[i], each);
+                        s_id[slot] = id.x;
+                        s_to[slot] = to;
+                        if (each == 2) {
+                            s_id[slot + 1] = id.y;
+                            s_to[slot + 1] = to + 1;
+                        }
+                    } else {  // no room left: straight to the list
+                        if (slot < kEmitBuffer) s_to[slot] = 0xFFFFFFFFu;
+                        const int q = atomicAdd(p.ecnt + i, each);
+                        int32_t* const dst = p.ebuf + (size_t)i * p.ecap;
+                        if (q < p.ecap) dst[q] = id.x;
+                        if (each == 2 && q + 1 < p.ecap) dst[q + 1] = id.y;
+                    }
                 }
             }
-            }
         }
+        __syncthreads();
+        if (s_n > kEmitBuffer / 2) flush();  // (the same in every thread)
     }
+    flush();
 }
 
 // kParts CTAs per lane.  Ids are distinct and in [0, m); CTA (lane, part)
