@@ -100,8 +100,8 @@ int core_limit_of(const iso_query_opts& o, int n) {
 
 // The sweep goes tile by tile (k_tiles) unless an option asks for one of the other
 // kernels or shapes the chunk schedule: the tiles were faster on every graph and
-// lane class measured (18M: 2.58 against 3.72 ms at 64 lanes, 0.89 against 1.27 at
-// one; 4M: 0.81 against 1.15 and 0.42 against 0.70).
+// lane class measured (18M: 2.45 against 3.72 ms at 64 lanes, 0.83 against 1.27 at
+// one; 1M: 0.31 against 0.48 and 0.21 against 0.35).
 bool wants_tiles(const iso_query_opts& o) {
     return o.sweep_kernel == 0 && o.threads_per_vertex == 0 && o.ctas_per_sm == 0 && o.fuse_width == 0 &&
            o.schedule_delay == 0 && o.solo_width == 0 && o.chunk_span == 0 && o.debug_stage_arcs == 0 &&

@@ -21,8 +21,9 @@
 // Bound: latency.  A tile of 50 vertices takes a CTA about 5 us, of which the rows
 // from outside are a third and five phases the rest (a phase: a serial chain of
 // shared-memory reads per four arcs of its largest vertex).  The sweep step (with
-// k_core) on 18M vertices, one GB300: 64 lanes 2.58 ms (chunk schedule 3.72), 16
-// lanes 1.30 (2.03), one lane 0.89 (1.27).
+// k_core) on 18M vertices, one GB300: 64 lanes 2.45 ms (chunk schedule 3.72), 32
+// lanes 1.66 (2.39), 16 lanes 1.25 (2.03), 8 lanes 1.12 (1.93), 4 lanes 0.92 (1.34),
+// one lane 0.83 (1.27); 1M: 64 lanes 0.31 (0.48), one lane 0.21 (0.35).
 #include "sweep_device.cuh"
 
 namespace {
@@ -85,8 +86,8 @@ __device__ __forceinline__ void st_lanes(uint32_t* row, const Place<K, TPV>& at,
     }
 }
 
-__device__ __forceinline__ void cp_async16(uint32_t* dst, const uint32_t* src) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(sa(dst)), "l"(src) : "memory");
+__device__ __forceinline__ void cp_async16(uint32_t dst, const uint32_t* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
 }
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
@@ -111,9 +112,15 @@ __host__ __device__ inline TileSmem tile_smem(const TileLimits& lim) {
     return s;
 }
 
+// Arcs a round of the sweep's inner loop.  With eight lanes a thread, the arithmetic
+// that spare arcs cost weighs more than the rounds (18M, 64 lanes: 2.51 ms with two,
+// 2.57 with four; 16 lanes 1.25 and 1.30); with one or four, the rounds' latency.
+__host__ __device__ constexpr int kTileArcs(int K) { return K >= 8 ? 2 : 4; }
+
 template <int K, int TPV>
 __global__ void __launch_bounds__(kThreads, kCtasPerSm) k_tiles(SweepParams p) {
     constexpr int LPT = K / TPV;
+    constexpr int ARCS = kTileArcs(K);
     static_assert(TPV == (int)sizeof(typename MaskOf<K>::T), "a thread writes one byte of the mask word");
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ unsigned long long full[2];
@@ -187,11 +194,23 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) k_tiles(SweepParams p) {
             const uint2* arcs = reinterpret_cast<const uint2*>(rec + rec[4]);
             const uint32_t* ext = rec + kTileHeader + phases;
             // rows from outside (final: written before the last grid barrier)
-            if constexpr (K >= 4) {
-                for (int i = tid; i < n_ext * (K / 4); i += kThreads)
-                    cp_async16(rows + 4 * i, p.d + (size_t)ext[i / (K / 4)] * K + 4 * (i % (K / 4)));
+            if constexpr (K >= 4) {  // a thread keeps to its piece of the rows
+                constexpr int Q = K / 4;
+                const uint32_t* const src = p.d + 4 * (tid % Q);
+                uint32_t dst = sa(rows) + 16u * (uint32_t)tid;
+#pragma unroll 4
+                for (int r = tid / Q; r < n_ext; r += kThreads / Q, dst += 16u * kThreads)
+                    cp_async16(dst, src + (size_t)ext[r] * K);
             } else {
-                for (int i = tid; i < n_ext; i += kThreads) rows[i] = __ldcg(p.d + ext[i]);
+                for (int i0 = tid; i0 < n_ext; i0 += 4 * kThreads) {  // four loads in flight
+                    uint32_t x[4];
+#pragma unroll
+                    for (int k = 0; k < 4; ++k)
+                        x[k] = i0 + k * kThreads < n_ext ? __ldcg(p.d + ext[i0 + k * kThreads]) : 0u;
+#pragma unroll
+                    for (int k = 0; k < 4; ++k)
+                        if (i0 + k * kThreads < n_ext) rows[i0 + k * kThreads] = x[k];
+                }
             }
             // the next tile's record
             if (tid == 0 && next_t < p.tiers) { fetch(b ^ 1); in_flight = true; }
@@ -199,15 +218,24 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) k_tiles(SweepParams p) {
             advance();
             // upward labels of own vertices: a row each, kInf in the lanes whose search did not get there
             bool up = false;
-            for (int i = tid; i < n_own; i += kThreads) {
-                const int v = (int)(vert[i].x & ~kTileStore);
-                int f = __ldcg(p.upflag + v);
-                if (f) {
-                    up = true;
-                    f = min(atomicAdd(&s_up, 1) + 1, kInPlace);
-                    if (f < kInPlace) s_up_v[f - 1] = v;
+            constexpr int FLAGS = K >= 32 ? 1 : 4;  // flags in flight per thread
+            for (int i0 = tid; i0 < n_own; i0 += FLAGS * kThreads) {
+                int v[FLAGS], f[FLAGS];
+#pragma unroll
+                for (int k = 0; k < FLAGS; ++k) {
+                    const int i = i0 + k * kThreads;
+                    v[k] = i < n_own ? (int)(vert[i].x & ~kTileStore) : -1;
+                    f[k] = v[k] >= 0 ? __ldcg(p.upflag + v[k]) : 0;
                 }
-                flags[i] = (uint8_t)f;
+#pragma unroll
+                for (int k = 0; k < FLAGS; ++k) {
+                    if (f[k]) {
+                        up = true;
+                        f[k] = min(atomicAdd(&s_up, 1) + 1, kInPlace);
+                        if (f[k] < kInPlace) s_up_v[f[k] - 1] = v[k];
+                    }
+                    if (v[k] >= 0) flags[i0 + k * kThreads] = (uint8_t)f[k];
+                }
             }
             if constexpr (K >= 4) cp_async_wait();
             up = __syncthreads_or(up);
@@ -237,78 +265,83 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) k_tiles(SweepParams p) {
             const uint32_t rows_a = sa(rows), arcs_a = sa(arcs);
             int hi = (int)rec[kTileHeader];
             int j = tid / TPV;  // (at most kThreads / TPV vertices a phase)
-            uint2 me = vert[min(j, n_own)];
-            uint32_t e = vert[min(j + 1, n_own)].y;
+            uint2 me = vert[j];  // (garbage from the record's later parts where j >= hi)
+            uint32_t e = vert[j + 1].y;
             for (int ph = 0; ph < phases; ++ph) {
-                const bool valid = j < hi;
-                const int v = (int)(me.x & ~kTileStore);
-                Lanes<LPT> acc;
+                if (j - lane / TPV < hi) {  // (uniform over the warp: some vertex is its)
+                    const bool valid = j < hi;
+                    const int v = (int)(me.x & ~kTileStore);
+                    Lanes<LPT> acc;
 #pragma unroll
-                for (int i = 0; i < LPT; ++i) acc.x[i] = kInf;
-                // Labels above tau need no clamp here: they only ever give labels above
-                // tau, and acc stays <= kInf, so that sums cannot wrap.
-                const uint32_t end = valid ? arcs_a + 8u * (e & 0xFFFFu) : 0u;
+                    for (int i = 0; i < LPT; ++i) acc.x[i] = kInf;
+                    // Labels above tau need no clamp here: they only ever give labels above
+                    // tau, and acc stays <= kInf, so that sums cannot wrap.
+                    const uint32_t end = valid ? arcs_a + 8u * (e & 0xFFFFu) : 0u;
 #pragma unroll 1
-                for (uint32_t a = arcs_a + 8u * (me.y & 0xFFFFu); a < end; a += 32u) {
-                    const uint4 q0 = lds128(a), q1 = lds128(a + 16u);
-                    const Lanes<LPT> r0 = lds_lanes<K, TPV>(rows_a + q0.x * (K * 4), at);
-                    const Lanes<LPT> r1 = lds_lanes<K, TPV>(rows_a + q0.z * (K * 4), at);
-                    const Lanes<LPT> r2 = lds_lanes<K, TPV>(rows_a + q1.x * (K * 4), at);
-                    const Lanes<LPT> r3 = lds_lanes<K, TPV>(rows_a + q1.z * (K * 4), at);
+                    for (uint32_t a = arcs_a + 8u * (me.y & 0xFFFFu); a < end; a += 8u * ARCS) {
+                        uint4 q[ARCS / 2];
+                        Lanes<LPT> r[ARCS];
 #pragma unroll
-                    for (int i = 0; i < LPT; ++i) acc.x[i] = __viaddmin_u32(r0.x[i], q0.y, acc.x[i]);
+                        for (int k = 0; k < ARCS / 2; ++k) q[k] = lds128(a + 16u * k);
 #pragma unroll
-                    for (int i = 0; i < LPT; ++i) acc.x[i] = __viaddmin_u32(r1.x[i], q0.w, acc.x[i]);
+                        for (int k = 0; k < ARCS / 2; ++k) {
+                            r[2 * k] = lds_lanes<K, TPV>(rows_a + q[k].x * (K * 4), at);
+                            r[2 * k + 1] = lds_lanes<K, TPV>(rows_a + q[k].z * (K * 4), at);
+                        }
 #pragma unroll
-                    for (int i = 0; i < LPT; ++i) acc.x[i] = __viaddmin_u32(r2.x[i], q1.y, acc.x[i]);
+                        for (int k = 0; k < ARCS / 2; ++k) {
 #pragma unroll
-                    for (int i = 0; i < LPT; ++i) acc.x[i] = __viaddmin_u32(r3.x[i], q1.w, acc.x[i]);
-                }
-                const int f = up && valid ? flags[j] : 0;
-                if (f == kInPlace) {  // only the lanes marked in upmask hold this batch's values
-                    const unsigned long long um = __ldcg(p.upmask + v);
+                            for (int i = 0; i < LPT; ++i) acc.x[i] = __viaddmin_u32(r[2 * k].x[i], q[k].y, acc.x[i]);
 #pragma unroll
-                    for (int i = 0; i < LPT; ++i) {
-                        const int l = at.lane_at(i);
-                        if ((um >> l) & 1ull) acc.x[i] = min(acc.x[i], __ldcg(p.d + (size_t)v * K + l));
+                            for (int i = 0; i < LPT; ++i) acc.x[i] = __viaddmin_u32(r[2 * k + 1].x[i], q[k].w, acc.x[i]);
+                        }
                     }
-                } else if (f) {
-                    const Lanes<LPT> r = lds_lanes<K, TPV>(rows_a + (uint32_t)(p.tile_lim.rows + f - 1) * (K * 4), at);
+                    const int f = up && valid ? flags[j] : 0;
+                    if (f == kInPlace) {  // only the lanes marked in upmask hold this batch's values
+                        const unsigned long long um = __ldcg(p.upmask + v);
 #pragma unroll
-                    for (int i = 0; i < LPT; ++i) acc.x[i] = min(acc.x[i], r.x[i]);
-                }
-                const uint32_t slot = me.y >> 16;
-                if (valid && slot != kTileNoRow) st_lanes<K, TPV>(rows + slot * K, at, acc);
-                // out-of-range bits: the sign of tau - label (both below 2^31), last element first
-                uint32_t bits = 0;
+                        for (int i = 0; i < LPT; ++i) {
+                            const int l = at.lane_at(i);
+                            if ((um >> l) & 1ull) acc.x[i] = min(acc.x[i], __ldcg(p.d + (size_t)v * K + l));
+                        }
+                    } else if (f) {
+                        const Lanes<LPT> r = lds_lanes<K, TPV>(rows_a + (uint32_t)(p.tile_lim.rows + f - 1) * (K * 4), at);
 #pragma unroll
-                for (int i = LPT - 1; i >= 0; --i) bits = __funnelshift_l(tau[i] - acc.x[i], bits, 1);
-                if (valid && ((me.x & kTileStore) || p.write_all)) {
-                    if (p.write_all) {  // distances are returned: out-of-range labels as kInf
-#pragma unroll
-                        for (int i = 0; i < LPT; ++i)
-                            if (acc.x[i] > tau[i]) acc.x[i] = kInf;
+                        for (int i = 0; i < LPT; ++i) acc.x[i] = min(acc.x[i], r.x[i]);
                     }
-                    st_lanes<K, TPV>(p.d + (size_t)v * K, at, acc);
+                    const uint32_t slot = me.y >> 16;
+                    if (valid && slot != kTileNoRow) st_lanes<K, TPV>(rows + slot * K, at, acc);
+                    // out-of-range bits: the sign of tau - label (both below 2^31), last element first
+                    uint32_t bits = 0;
+#pragma unroll
+                    for (int i = LPT - 1; i >= 0; --i) bits = __funnelshift_l(tau[i] - acc.x[i], bits, 1);
+                    if (valid && ((me.x & kTileStore) || p.write_all)) {
+                        if (p.write_all) {  // distances are returned: out-of-range labels as kInf
+#pragma unroll
+                            for (int i = 0; i < LPT; ++i)
+                                if (acc.x[i] > tau[i]) acc.x[i] = kInf;
+                        }
+                        st_lanes<K, TPV>(p.d + (size_t)v * K, at, acc);
+                    }
+                    // one byte of the mask word per thread: with two quads, a thread and its
+                    // neighbour swap a nibble each, the even one gets the lower quads' byte
+                    bits = ~bits;
+                    int byte = sub;
+                    if constexpr (LPT == 8) {
+                        if (at.o1 > at.o2) bits = (bits >> 4 & 0xFu) | bits << 4;  // lower quad first
+                    }
+                    if constexpr (LPT == 8 && TPV > 1) {
+                        const uint32_t other = __shfl_xor_sync(0xffffffffu, bits, 1);
+                        bits = sub & 1 ? (other >> 4 & 0xFu) | (bits & 0xF0u) : (bits & 0xFu) | (other & 0xFu) << 4;
+                        byte = sub / 2 + (sub & 1) * (TPV / 2);
+                    }
+                    if (valid) static_cast<uint8_t*>(p.mask)[(size_t)v * TPV + byte] = (uint8_t)(bits & ((1u << LPT) - 1u));
                 }
-                // one byte of the mask word per thread: with two quads, a thread and its
-                // neighbour swap a nibble each, the even one gets the lower quads' byte
-                bits = ~bits;
-                int byte = sub;
-                if constexpr (LPT == 8) {
-                    if (at.o1 > at.o2) bits = (bits >> 4 & 0xFu) | bits << 4;  // lower quad first
-                }
-                if constexpr (LPT == 8 && TPV > 1) {
-                    const uint32_t other = __shfl_xor_sync(0xffffffffu, bits, 1);
-                    bits = sub & 1 ? (other >> 4 & 0xFu) | (bits & 0xF0u) : (bits & 0xFu) | (other & 0xFu) << 4;
-                    byte = sub / 2 + (sub & 1) * (TPV / 2);
-                }
-                if (valid) static_cast<uint8_t*>(p.mask)[(size_t)v * TPV + byte] = (uint8_t)(bits & ((1u << LPT) - 1u));
                 if (ph + 1 < phases) {
                     j = hi + tid / TPV;
                     hi = (int)rec[kTileHeader + ph + 1];
-                    me = vert[min(j, n_own)];
-                    e = vert[min(j + 1, n_own)].y;
+                    me = vert[j];
+                    e = vert[j + 1].y;
                 }
                 __syncthreads();
             }
@@ -370,19 +403,21 @@ cudaError_t launch(const SweepParams& p, int grid, cudaStream_t s) {
 TileLimits iso_tile_limits(int K) {
     // Five CTAs per SM (about 43 KB each): a tile costs mostly latency (rows from
     // outside 1.4 us, 0.5 us a phase), so tiles in flight count for more than large
-    // tiles.  18M vertices, 64 lanes, ms of the whole sweep step: rows 100 (5 CTAs)
-    // 2.58, 120 2.61, 156 (4 CTAs) 2.71; comp 16 2.58, 12 2.58, 8 2.64.  16 lanes:
-    // rows 300 1.30, 220 1.41, 400 1.32; comp 16 1.30, 8 1.33, 32 1.33.  One lane:
-    // 1,500 rows and 16 KB 0.89 (comp 32; 16: 0.95), 1,000 and 10 KB 0.93.
+    // tiles, except with one lane, where a tile's own work is small.  18M vertices,
+    // ms of the whole sweep step: 64 lanes, rows 100 (5 CTAs) 2.58, 120 2.61, 156
+    // (4 CTAs) 2.71, 80 (6 CTAs) 2.62; comp 16 2.58, 12 2.58, 8 2.64.  16 lanes: rows
+    // 300 1.25, 400 1.27, 220 1.35.  8 lanes: rows 400 1.12, 600 1.14.  One lane: 24 KB
+    // records 0.83, 16 KB 0.89, 10 KB 0.90.
     TileLimits l{};
     switch (K) {
         case 64: l.rows = 100; l.blob_bytes = 6144; l.comp = 16; break;
         case 32: l.rows = 200; l.blob_bytes = 8192; l.comp = 16; break;
         case 16: l.rows = 300; l.blob_bytes = 10240; l.comp = 16; break;
-        case 8: l.rows = 600; l.blob_bytes = 12288; l.comp = 24; break;
+        case 8: l.rows = 400; l.blob_bytes = 10240; l.comp = 24; break;
         case 4: l.rows = 1000; l.blob_bytes = 14336; l.comp = 32; break;
-        default: l.rows = 1500; l.blob_bytes = 16384; l.comp = 32; break;
+        default: l.rows = 2500; l.blob_bytes = 24576; l.comp = 32; break;
     }
+    l.arcs = kTileArcs(K);
     l.width = kThreads / (K >= 8 ? K / 8 : 1);
     return l;
 }

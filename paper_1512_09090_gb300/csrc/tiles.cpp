@@ -87,7 +87,7 @@ struct Job {
 int iso_make_tiles(int n, int L, const int32_t* level_off, const uint32_t* down_off, const int32_t* down_src,
                    const int32_t* down_len, const int32_t* bfs, int core_n, const TileLimits& lim, TilePlan* out) {
     if (n <= 0 || L <= 0 || core_n < 0 || core_n > n || lim.rows < 2 || lim.rows >= (int)kTileNoRow || lim.comp < 1 ||
-        lim.width < 1 ||
+        lim.width < 1 || (lim.arcs != 2 && lim.arcs != 4) ||
         lim.blob_bytes < 64)
         return -1;
     const uint32_t m = down_off[n];
@@ -237,7 +237,7 @@ int iso_make_tiles(int n, int L, const int32_t* level_off, const uint32_t* down_
                     if (done[c]) continue;
                     fresh.clear();
                     int in = 0;
-                    int64_t ca = 0;  // (a multiple of four for each vertex)
+                    int64_t ca = 0;  // (a multiple of lim.arcs for each vertex)
                     for (int32_t i = coff[c]; i < coff[c + 1]; ++i) {
                         const int32_t v = cver[i];
                         for (uint32_t s = so[v]; s < so[v + 1]; ++s)
@@ -249,7 +249,7 @@ int iso_make_tiles(int n, int L, const int32_t* level_off, const uint32_t* down_
                             const int32_t u = down_src[a];
                             if (comp[u] != c && !ext.has(u)) { ext.add(u); fresh.push_back(u); }
                         }
-                        ca = (ca + 3) & ~(int64_t)3;
+                        ca = (ca + lim.arcs - 1) / lim.arcs * lim.arcs;
                     }
                     const int64_t n_own = (int64_t)own.size() + coff[c + 1] - coff[c];
                     // (phases: full ones, and others that each shorten the longest path; three gaps)
@@ -353,7 +353,7 @@ int iso_make_tiles(int n, int L, const int32_t* level_off, const uint32_t* down_
                         w.push_back((uint32_t)down_len[a]);
                         ++at;
                     }
-                    for (; at & 3; ++at) {  // the last arc's row again
+                    for (; at % (uint32_t)lim.arcs; ++at) {  // the last arc's row again
                         w.push_back(w[w.size() - 2]);
                         w.push_back(kNever);
                     }

@@ -11,6 +11,7 @@ struct TileLimits {
     int blob_bytes;  // the tile's record (a multiple of 16)
     int comp;        // vertices of a component
     int width;       // vertices of a phase: what the CTA sweeps at once
+    int arcs;        // a vertex's arcs are padded to a multiple of this (2 or 4)
 };
 
 // A tile's record, in 32-bit words (16-byte aligned and padded, one bulk copy):
@@ -22,8 +23,8 @@ struct TileLimits {
 //     {sweep position | kTileStore if another tile reads its row,
 //      first arc | row << 16 (kTileNoRow: no own vertex of the tile reads it)}
 //   arcs of two words: {source row, length}, grouped by own vertex, a multiple of
-//   four for each (16-byte aligned): spare ones have length 0x7FFFFFFF, which
-//   never lowers a label, and the row of the arc before them
+//   lim.arcs for each: a spare one has length 0x7FFFFFFF, which never lowers a
+//   label, and the row of the arc before it
 constexpr int kTileHeader = 8;
 constexpr uint32_t kTileStore = 0x80000000u;
 constexpr uint32_t kTileNoRow = 0xFFFFu;

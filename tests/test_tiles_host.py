@@ -104,7 +104,7 @@ DRIVER = textwrap.dedent(r"""
                     const uint32_t a0 = vert[2 * j + 1] & 0xFFFFu, a1 = vert[2 * j + 3] & 0xFFFFu;
                     for (uint32_t a = a0; a < a1; ++a) {
                         const uint32_t s = arc[2 * a];
-                        if (a0 % 4 || a1 % 4) return fail("arcs in fours", q, a);
+                        if (a0 % lim.arcs || a1 % lim.arcs) return fail("padded arcs", q, a);
                         if ((int)s >= lim.rows || row_phase[s] >= phase) return fail("row of a later phase", q, s);
                         x = std::min(x, row[s] + arc[2 * a + 1]);
                     }
@@ -135,14 +135,14 @@ DRIVER = textwrap.dedent(r"""
     }
 
     int main() {
-        const TileLimits sizes[] = {{200, 8192, 32, 16}, {24, 768, 4, 3}, {12, 640, 1, 1}, {3000, 32768, 64, 128}};
+        const TileLimits sizes[] = {{200, 8192, 32, 16, 2}, {24, 768, 4, 3, 4}, {12, 640, 1, 1, 4}, {3000, 32768, 64, 128, 4}};
         for (unsigned seed = 1; seed <= 60; ++seed)
             for (const TileLimits& lim : sizes)
                 for (int local = 0; local < 2; ++local)
                     if (check(seed, local, (int)(seed % 4), lim, false)) return 1;
         // a vertex with more sources than a tile has rows: no plan
         int none = 0;
-        for (unsigned seed = 1; seed <= 20; ++seed) none += check(seed, 0, 0, TileLimits{2, 64, 1, 8}, true);
+        for (unsigned seed = 1; seed <= 20; ++seed) none += check(seed, 0, 0, TileLimits{2, 64, 1, 8, 2}, true);
         if (none) return 1;
         std::printf("OK\n");
         return 0;
