@@ -1273,6 +1273,7 @@ int iso_graph_view_of(const iso_graph* g, iso_graph_view* v) {
     v->down_arc = g->down_arc; v->up_arc = g->up_arc;
     v->pair_head = g->pair_head; v->pair_ids = g->pair_ids; v->pos = g->pos; v->level_off = g->level_off;
     v->pair_owner = g->pair_owner;
+    v->core_arc = g->core_arc; v->level_arc = g->level_arc;
     v->h_level_off = g->h_level_off.data();
     return ISO_OK;
 }

@@ -6,7 +6,7 @@
 // a latency-critical thread that must not wait on allocator locks or on the
 // device-wide synchronisation a cudaFree can imply, or an embedding host that
 // forbids allocation after start-up.  For them this entry point runs the same
-// kernels (upward search, sweep, emission, sort) on slices of g_scratch, a
+// kernels (upward search, core, plain sweep, emission, sort) on slices of g_scratch, a
 // static __device__ array of fixed size.  Every GPU that loads the library holds
 // that array until the process exits.
 //
@@ -44,6 +44,11 @@ constexpr int kMaxLevels = 4096;
 constexpr int kUpCap = 16384;                        // global table slots per lane
 constexpr int kMaxUpward = kUpCap / 2;
 constexpr int kMaxArcs = ISO_NOALLOC_MAX_ARCS;       // isochrone edges per query
+// The top of the hierarchy, at most this many vertices, is swept per lane by one CTA
+// (k_core): its blocks cost 1 us each there and 7 us each as grid-wide steps (1M
+// vertices: 112 of 130 blocks; four queries 1.04 ms without a core, now 0.59).
+constexpr int kCore = 20000;
+static_assert(kCore <= kCoreMaxVertices && kCore <= kMaxArcs, "the core's labels take the sort's scratch");
 
 // Byte offsets of the slices (each 256-byte aligned).
 constexpr size_t al(size_t x) { return (x + 255) & ~(size_t)255; }
@@ -165,10 +170,12 @@ extern "C" int iso_query_noalloc(iso_graph* g, int32_t k, const int32_t* sources
     if ((e = cudaMemsetAsync(ctl, 0, kCtlWords * 4, stream)) != cudaSuccess ||
         (e = cudaMemsetAsync(base + kOffFlag, 0, (size_t)gv.n, stream)) != cudaSuccess)
         return fail_enqueued(ISO_E_CUDA, "clearing scratch", e, stream);
-    // one grid-wide step per level
-    for (int j = 0; j < gv.L; ++j) g_sched[j] = make_int4(kStepWide, j, j + 1, 0);
-    if ((e = cudaMemcpyAsync(base + kOffSched, g_sched, (size_t)gv.L * sizeof(int4), cudaMemcpyHostToDevice,
-                             stream)) != cudaSuccess)
+    // the per-lane core, then one grid-wide step per level
+    int core = 0;
+    while (core < gv.L && core < kCoreMaxLevels && gv.h_level_off[core + 1] <= kCore) ++core;
+    for (int j = core; j < gv.L; ++j) g_sched[j - core] = make_int4(kStepWide, j, j + 1, 0);
+    if (core < gv.L && (e = cudaMemcpyAsync(base + kOffSched, g_sched, (size_t)(gv.L - core) * sizeof(int4),
+                                            cudaMemcpyHostToDevice, stream)) != cudaSuccess)
         return fail_enqueued(ISO_E_CUDA, "schedule copy", e, stream);
 
     UpParams up{};
@@ -182,7 +189,12 @@ extern "C" int iso_query_noalloc(iso_graph* g, int32_t k, const int32_t* sources
     sw.sched = (const int4*)(base + kOffSched); sw.pairs = up.pairs; sw.cnt = up.cnt; sw.tau = io + kLanes;
     sw.d = (uint32_t*)(base + kOffD); sw.mask = base + kOffMask; sw.upflag = base + kOffFlag;
     sw.bar = (uint32_t*)(ctl + 4); sw.status = ctl; sw.timeout_ns = 2000000000LL; sw.n = gv.n; sw.L = gv.L;
-    sw.nsched = gv.L; sw.cap = kUpCap; sw.last_level_block = gv.L - 1; sw.write_all = 0; sw.bar_extra = 0;
+    sw.nsched = gv.L - core; sw.cap = kUpCap; sw.last_level_block = gv.L - 1; sw.write_all = 0; sw.bar_extra = 0;
+    sw.core_levels = core; sw.core_n = gv.h_level_off[core];
+    sw.core_arc = gv.core_arc; sw.level_arc = gv.level_arc;
+    sw.core_out = (uint32_t*)(base + kOffTmp);  // (the sort uses this slice after the sweep)
+    if (core > 0 && (e = iso_launch_core(sw, kLanes, stream)) != cudaSuccess)
+        return fail_enqueued(ISO_E_CUDA, "core launch", e, stream);
     int block = 0;
     const int occ = iso_sweep_occupancy(kLanes, 1, &block);
     if (occ <= 0) return fail_enqueued(ISO_E_CUDA, "sweep kernel cannot be resident", cudaGetLastError(), stream);

@@ -52,7 +52,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_core(SweepParams p) {
     const int2* pr = p.pairs + (size_t)b * p.cap;
     for (int i = tid; i < np; i += kThreads) {
         const int2 q = pr[i];
-        lab[q.x] = (uint32_t)q.y;
+        if (q.x < cn) lab[q.x] = (uint32_t)q.y;  // (the plain sweep's lists hold all upward labels)
     }
     __syncthreads();
     // first arcs of levels j (pre0) and j + 1 (pre1), read two levels ahead

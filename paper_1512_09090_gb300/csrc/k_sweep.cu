@@ -17,58 +17,13 @@
 // earlier in the same launch are read with ld.global.cg so no SM can hit a stale
 // L1 line.  Every barrier wait is bounded by a time limit after which the
 // kernel records kStTimeout and returns.
-#include <cooperative_groups.h>
-
-#include "iso_device.cuh"
+#include "sweep_device.cuh"
 
 namespace {
 
 using namespace isod;
 
 constexpr int kThreads = 512;
-
-template <int K> struct MaskOf { using T = uint8_t; };
-template <> struct MaskOf<16> { using T = uint16_t; };
-template <> struct MaskOf<32> { using T = uint32_t; };
-template <> struct MaskOf<64> { using T = unsigned long long; };
-
-__device__ bool grid_sync(const SweepParams& p) {
-    __shared__ int s_ok;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int ok = 1;
-        volatile int32_t* st = p.status;
-        volatile uint32_t* gen = p.bar + 1;
-        if (*st != kStOk) {
-            ok = 0;
-        } else {
-            const uint32_t g0 = *gen;
-            __threadfence();
-            const uint32_t want = gridDim.x + (uint32_t)p.bar_extra;
-            if (atomicAdd(p.bar, 1u) + 1u == want) {
-                atomicExch(p.bar, 0u);
-                __threadfence();
-                atomicAdd(p.bar + 1, 1u);
-            } else {
-                const unsigned long long t0 = global_ns();
-                const unsigned long long max_iter = (unsigned long long)p.timeout_ns / 16 + 4096;
-                for (unsigned long long it = 0; *gen == g0; ++it) {
-                    if (*st != kStOk) { ok = 0; break; }
-                    if (global_ns() - t0 > (unsigned long long)p.timeout_ns || it > max_iter) {
-                        atomicCAS(p.status, kStOk, kStTimeout);
-                        ok = 0;
-                        break;
-                    }
-                    __nanosleep(32);
-                }
-            }
-            __threadfence();
-        }
-        s_ok = ok;
-    }
-    __syncthreads();
-    return s_ok != 0;
-}
 
 template <int LPT> struct Row { uint32_t x[LPT]; };
 
@@ -190,6 +145,7 @@ __global__ void __launch_bounds__(kThreads) k_sweep(SweepParams p) {
         const int2* pr = p.pairs + (size_t)lane * p.cap;
         for (size_t j = gtid; j < (size_t)c; j += gsz) {
             const int v = pr[j].x;
+            if (v < p.core_n) continue;
             uint32_t* row = p.d + (size_t)v * K;
             if constexpr (K >= 4) {
 #pragma unroll
@@ -200,12 +156,15 @@ __global__ void __launch_bounds__(kThreads) k_sweep(SweepParams p) {
             p.upflag[v] = 1;
         }
     }
+    // labels of the per-lane core, if k_core has swept one
+    if (p.core_levels > 0) core_rows<K, kThreads>(p, tid);
     if (!grid_sync(p)) return;
     for (int lane = 0; lane < K; ++lane) {
         const int c = p.cnt[lane];
         const int2* pr = p.pairs + (size_t)lane * p.cap;
         for (size_t j = gtid; j < (size_t)c; j += gsz) {
             const int2 q = pr[j];
+            if (q.x < p.core_n) continue;
             atomicMin(p.d + (size_t)q.x * K + lane, (uint32_t)q.y);
         }
     }
