@@ -577,8 +577,6 @@ int enqueue(iso_workspace* ws, bool want_dist, bool capturing) {
     ga.ebuf = ws->ebuf; ga.ecnt = ws->ecnt(); ga.tmp = ws->tmp; ga.out = ws->out; ga.out_off = ws->out_off;
     ga.k = K; ga.ecap = ws->ecap;
     ga.status = ws->status();
-    ga.key_bits = 1;
-    while (ga.key_bits < 31 && (int64_t(1) << ga.key_bits) < g->m) ++ga.key_bits;
     ga.m = g->m;
     ISO_CK(iso_launch_sort_gather(ga, K, s));
     if (want_dist) {

@@ -158,8 +158,9 @@ struct GatherParams {
     int32_t* out;              // contiguous lists
     int64_t* out_off;          // [K+1]
     int k, ecap;
-    int key_bits;              // bits needed for arc ids
     int64_t m;                 // arc ids are in [0, m)
+    int part_bits;             // (set by the launcher) log2 of the CTAs per lane ...
+    uint32_t mult;             // ... and 2^46 / m, or 0 where m <= 2^14
     const int32_t* status;     // batch status: nothing is written once it is not kStOk
 };
 

@@ -6,7 +6,7 @@
 // for about a thousand of them.
 //
 // Then k_sort_gather sorts each lane's ids ascending (bucket sort in shared
-// memory, four CTAs per lane) and writes them to the contiguous output at the
+// memory, several CTAs per lane) and writes them to the contiguous output at the
 // lane's offset; CTA 0 also writes the offsets.
 #include "iso_device.cuh"
 
@@ -131,75 +131,141 @@ __global__ void __launch_bounds__(kEmitThreads) k_emit(EmitParams p) {
     flush();
 }
 
-// kParts CTAs per lane.  Ids are distinct and in [0, m); CTA (lane, part)
-// takes the ids of the part-th of kParts equal slices of [0, m) (their count
-// and the counts of the slices before it come from one pass over the lane's
-// list), so the parts' sorted lists are consecutive pieces of the lane's
-// sorted list.  A part is split into about cnt/4 equal buckets of its slice
-// (histogram, scan, scatter into shared memory); buckets are then sorted on
-// their own: small ones by one thread each (insertion sort), any bucket above
-// kSmallBucket ids by the whole CTA (every id's rank by counting the smaller
-// ones in its bucket, written straight to its place).  CTA 0 also writes the
-// offsets of all lanes.  A lane one of whose parts would not fit shared memory
-// is sorted by its part-0 CTA alone with the list in global memory (the other
-// parts of that lane return).
+// `parts` CTAs per lane (the fewer lanes, the more).  Ids are distinct and in
+// [0, m); fine(id) maps them to [0, 2^14) without ever decreasing (one
+// multiplication; below 2^14 ids it is the id itself), its top bits are the part
+// and the next ones a bucket of the part.  CTA (lane, part) reads the lane's list
+// twice: to count the ids of every part and of its own buckets, and, after a scan,
+// to scatter its own ids into their buckets in shared memory.  Small buckets
+// (about four ids) are then sorted by one thread each (insertion sort), larger
+// ones by the whole CTA (every id's place is the number of smaller ids in its
+// bucket).  The parts' sorted lists are consecutive pieces of the lane's.  CTA 0
+// also writes the offsets.  A lane one of whose parts would not fit shared memory
+// is sorted by its part-0 CTA alone with the list in global memory.
+//
+// Bound by latency (5 MB of ids): two passes over the longest list.  18M vertices,
+// 64 queries (1.2M ids): 0.20 ms with three passes, two 64-bit divisions an id and
+// a ten-step scan, now 0.057; one query (15,000 ids) 0.061 with four CTAs, now 0.024.
+constexpr int kFineBits = 14;
 constexpr int kMaxBuckets = 4096;
 constexpr int kSmallBucket = 64;
 constexpr int kMaxBigBuckets = 256;  // big buckets listed for the whole-CTA ranking
-constexpr int kParts = 4;
+constexpr int kMaxParts = 16;
 
-// Sorts the ids x of src[0..src_cnt) with lo <= x < hi (cnt of them) into
-// out[0..cnt): bucketed into B[0..cnt) by equal slices of [lo, hi) (about four
-// ids per bucket), small buckets sorted in place and copied, big buckets
-// ranked straight into out.
-__device__ void bucket_sort(const int32_t* src, int src_cnt, int32_t* B, int cnt, int32_t* out, int64_t lo,
-                            int64_t hi, int32_t* s_hist, int32_t* s_cur) {
-    __shared__ int s_part[kSortThreads];
-    __shared__ int s_nbig, s_big[kMaxBigBuckets];
-    int lg = 0;
-    while ((1 << lg) < kMaxBuckets && (4 << lg) < cnt) ++lg;
-    const int nb = 1 << lg;
-    const uint64_t span = (uint64_t)(hi - lo);
-    auto bucket_of = [&](int32_t x) { return (int)((uint64_t)(x - lo) * (uint64_t)nb / span); };
-    auto mine = [&](int32_t x) { return x >= lo && x < hi; };
-    for (int bb = threadIdx.x; bb <= nb; bb += blockDim.x) s_hist[bb] = 0;
-    if (threadIdx.x == 0) s_nbig = 0;
-    __syncthreads();
-    for (int i = threadIdx.x; i < src_cnt; i += blockDim.x) {
-        const int32_t x = src[i];
-        if (mine(x)) atomicAdd(&s_hist[bucket_of(x)], 1);
-    }
-    __syncthreads();
-    // exclusive scan of the nb counts (nb <= kMaxBuckets, a few per thread)
-    {
-        const int per = (nb + blockDim.x - 1) / blockDim.x;
-        const int b0 = threadIdx.x * per;
-        int sum = 0;
-        for (int bb = b0; bb < min(b0 + per, nb); ++bb) sum += s_hist[bb];
-        s_part[threadIdx.x] = sum;
-        __syncthreads();
-        for (int o = 1; o < (int)blockDim.x; o <<= 1) {
-            const int v = threadIdx.x >= (unsigned)o ? s_part[threadIdx.x - o] : 0;
-            __syncthreads();
-            s_part[threadIdx.x] += v;
-            __syncthreads();
+__device__ __forceinline__ uint32_t fine_of(uint32_t id, uint32_t mult) { return mult ? __umulhi(id, mult) : id; }
+
+__global__ void __launch_bounds__(kSortThreads) k_sort_gather(GatherParams p) {
+    extern __shared__ int32_t sbuf[];
+    int32_t* s_hist = sbuf + kSortSmem;           // [kMaxBuckets + 1]
+    int32_t* s_cur = s_hist + kMaxBuckets + 1;    // [kMaxBuckets]
+    __shared__ long long s_off;
+    __shared__ int s_pc[kMaxParts], s_warp[kSortThreads / 32], s_nbig, s_big[kMaxBigBuckets];
+    const int lane = blockIdx.x >> p.part_bits;
+    int part = (int)blockIdx.x & ((1 << p.part_bits) - 1);
+    const int tid = threadIdx.x, warp = tid >> 5, wl = tid & 31;
+    if (*(volatile const int32_t*)p.status != kStOk) return;  // failed batch: the host reports it
+    // list sizes and offsets (at most 64 lanes): two lanes a thread of warp 0
+    if (warp == 0) {
+        const long long c0 = 2 * wl < p.k ? min(p.ecnt[2 * wl], p.ecap) : 0;
+        const long long c1 = 2 * wl + 1 < p.k ? min(p.ecnt[2 * wl + 1], p.ecap) : 0;
+        long long sum = c0 + c1;
+        for (int o = 1; o < 32; o <<= 1) {
+            const long long up = __shfl_up_sync(0xffffffffu, sum, o);
+            if (wl >= o) sum += up;
         }
-        int acc = s_part[threadIdx.x] - sum;
-        for (int bb = b0; bb < min(b0 + per, nb); ++bb) {
-            const int c = s_hist[bb];
-            s_hist[bb] = acc;
-            s_cur[bb] = acc;
+        if (blockIdx.x == 0) {
+            if (wl == 0) p.out_off[0] = 0;
+            if (2 * wl < p.k) p.out_off[2 * wl + 1] = sum - c1;
+            if (2 * wl + 1 < p.k) p.out_off[2 * wl + 2] = sum;
+        }
+        if (lane / 2 == wl) s_off = lane & 1 ? sum - c1 : sum - c1 - c0;
+    }
+    if (tid < kMaxParts) s_pc[tid] = 0;
+    if (tid == 0) s_nbig = 0;
+    if (lane >= p.k) return;
+    const int cnt = min(p.ecnt[lane], p.ecap);
+    if (cnt == 0) return;
+    const int32_t* seg = p.ebuf + (size_t)lane * p.ecap;
+    // buckets per part: about four ids each if the parts are alike
+    int lg = 0;
+    while (lg < kFineBits - p.part_bits && (1 << lg) < kMaxBuckets && (4ll << (lg + p.part_bits)) < cnt) ++lg;
+    int pbits = p.part_bits;
+    int32_t* B = sbuf;
+    int my = 0, below = 0;
+    for (int pass = 0;; ++pass) {
+        // (second pass: a part is too large, the lane is sorted as one by this CTA)
+        const int nb = 1 << lg, shift = kFineBits - pbits - lg;
+        for (int i = tid; i < nb; i += kSortThreads) s_hist[i] = 0;
+        __syncthreads();
+        for (int i0 = tid; i0 < cnt; i0 += 4 * kSortThreads) {
+            uint32_t x[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) x[k] = i0 + k * kSortThreads < cnt ? (uint32_t)seg[i0 + k * kSortThreads] : 0u;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                if (i0 + k * kSortThreads >= cnt) break;
+                const int f = (int)fine_of(x[k], p.mult) >> shift, q = f >> lg;
+                if (q == part) atomicAdd(&s_hist[f & (nb - 1)], 1);
+                // the other parts' counts: one atomic per warp and part
+                if (pass == 0) {
+                    const unsigned peers = __match_any_sync(__activemask(), q);
+                    if (wl == __ffs(peers) - 1) atomicAdd(&s_pc[q], __popc(peers));
+                }
+            }
+        }
+        __syncthreads();
+        if (pass == 1) { my = cnt; below = 0; break; }
+        bool whole = false;
+        for (int q = 0; q < (1 << pbits); ++q) {
+            whole = whole || s_pc[q] > kSortSmem;
+            if (q < part) below += s_pc[q];
+        }
+        my = s_pc[part];
+        if (!whole) break;
+        if (part != 0) return;
+        B = p.tmp + (size_t)lane * p.ecap;
+        pbits = 0;
+        lg = 12;
+        __syncthreads();
+    }
+    if (my == 0) return;
+    const int nb = 1 << lg, shift = kFineBits - pbits - lg;
+    int32_t* out = p.out + s_off + below;
+    // exclusive scan of the nb counts (nb <= kMaxBuckets, at most four per thread)
+    {
+        const int per = (nb + kSortThreads - 1) / kSortThreads, b0 = tid * per;
+        int sum = 0;
+        for (int i = b0; i < min(b0 + per, nb); ++i) sum += s_hist[i];
+        int run = sum;
+        for (int o = 1; o < 32; o <<= 1) {
+            const int up = __shfl_up_sync(0xffffffffu, run, o);
+            if (wl >= o) run += up;
+        }
+        if (wl == 31) s_warp[warp] = run;
+        __syncthreads();
+        int acc = run - sum;
+        for (int w = 0; w < warp; ++w) acc += s_warp[w];
+        for (int i = b0; i < min(b0 + per, nb); ++i) {
+            const int c = s_hist[i];
+            s_hist[i] = acc;
+            s_cur[i] = acc;
             acc += c;
         }
-        if (threadIdx.x == 0) s_hist[nb] = cnt;
+        if (tid == 0) s_hist[nb] = my;
     }
     __syncthreads();
-    for (int i = threadIdx.x; i < src_cnt; i += blockDim.x) {
-        const int32_t x = src[i];
-        if (mine(x)) B[atomicAdd(&s_cur[bucket_of(x)], 1)] = x;
+    for (int i0 = tid; i0 < cnt; i0 += 4 * kSortThreads) {
+        uint32_t x[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) x[k] = i0 + k * kSortThreads < cnt ? (uint32_t)seg[i0 + k * kSortThreads] : 0u;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int f = (int)fine_of(x[k], p.mult) >> shift;
+            if (i0 + k * kSortThreads < cnt && f >> lg == part) B[atomicAdd(&s_cur[f & (nb - 1)], 1)] = (int32_t)x[k];
+        }
     }
     __syncthreads();
-    for (int bb = threadIdx.x; bb < nb; bb += blockDim.x) {
+    for (int bb = tid; bb < nb; bb += kSortThreads) {
         const int blo = s_hist[bb], bhi = s_hist[bb + 1];
         if (bhi - blo > kSmallBucket) {
             const int q = atomicAdd(&s_nbig, 1);
@@ -212,75 +278,29 @@ __device__ void bucket_sort(const int32_t* src, int src_cnt, int32_t* B, int cnt
             while (j >= blo && B[j] > x) { B[j + 1] = B[j]; --j; }
             B[j + 1] = x;
         }
-        for (int i = blo; i < bhi; ++i) out[i] = B[i];
     }
     __syncthreads();
-    // big buckets: the whole CTA, each id's place is the count of smaller ids
-    // (the list of them, or every bucket if it overflowed)
+    // sorted buckets go out together (coalesced); big ones are ranked by the whole
+    // CTA, from the list of them or, if it overflowed, bucket by bucket
     const int nbig = s_nbig;
+    if (nbig == 0) {
+        for (int i = tid; i < my; i += kSortThreads) out[i] = B[i];
+        return;
+    }
+    for (int bb = tid; bb < nb; bb += kSortThreads)
+        if (s_hist[bb + 1] - s_hist[bb] <= kSmallBucket)
+            for (int i = s_hist[bb]; i < s_hist[bb + 1]; ++i) out[i] = B[i];
     for (int t = 0; t < (nbig <= kMaxBigBuckets ? nbig : nb); ++t) {
         const int bb = nbig <= kMaxBigBuckets ? s_big[t] : t;
         const int blo = s_hist[bb], bhi = s_hist[bb + 1];
         if (bhi - blo <= kSmallBucket) continue;
-        for (int i = blo + threadIdx.x; i < bhi; i += blockDim.x) {
+        for (int i = blo + tid; i < bhi; i += kSortThreads) {
             const int32_t x = B[i];
             int r = 0;
             for (int j = blo; j < bhi; ++j) r += B[j] < x;
             out[blo + r] = x;
         }
     }
-}
-
-__global__ void __launch_bounds__(kSortThreads) k_sort_gather(GatherParams p) {
-    extern __shared__ int32_t sbuf[];
-    int32_t* s_hist = sbuf + kSortSmem;           // [kMaxBuckets + 1]
-    int32_t* s_cur = s_hist + kMaxBuckets + 1;    // [kMaxBuckets]
-    __shared__ long long s_off;
-    __shared__ int s_pc[kParts];
-    const int lane = blockIdx.x / kParts, part = blockIdx.x % kParts;
-    if (*(volatile const int32_t*)p.status != kStOk) return;  // failed batch: the host reports it
-    if (threadIdx.x == 0) {
-        long long off = 0;
-        for (int i = 0; i < lane; ++i) off += min(p.ecnt[i], p.ecap);
-        s_off = off;
-        if (blockIdx.x == 0) {
-            long long o = 0;
-            p.out_off[0] = 0;
-            for (int i = 0; i < p.k; ++i) { o += min(p.ecnt[i], p.ecap); p.out_off[i + 1] = o; }
-        }
-    }
-    if (threadIdx.x < kParts) s_pc[threadIdx.x] = 0;
-    __syncthreads();
-    if (lane >= p.k) return;
-    const int cnt = min(p.ecnt[lane], p.ecap);
-    if (cnt == 0) return;
-    const int32_t* seg = p.ebuf + (size_t)lane * p.ecap;
-    int32_t* out = p.out + s_off;
-    const int64_t m = p.m > 0 ? p.m : 1;
-    // part q holds [slice(q), slice(q + 1)), i.e. exactly the ids x with x * kParts / m == q
-    auto slice = [&](int q) { return (m * q + kParts - 1) / kParts; };
-    {
-        int c[kParts] = {0, 0, 0, 0};
-        for (int i = threadIdx.x; i < cnt; i += blockDim.x)
-            c[min((int)((int64_t)seg[i] * kParts / m), kParts - 1)]++;
-        for (int q = 0; q < kParts; ++q)
-            if (c[q]) atomicAdd(&s_pc[q], c[q]);
-    }
-    __syncthreads();
-    bool lane_mode = false;
-    int below = 0;
-    for (int q = 0; q < kParts; ++q) {
-        lane_mode = lane_mode || s_pc[q] > kSortSmem;
-        if (q < part) below += s_pc[q];
-    }
-    if (!lane_mode) {
-        const int my = s_pc[part];
-        if (my > 0) bucket_sort(seg, cnt, sbuf, my, out + below, slice(part), slice(part + 1), s_hist, s_cur);
-        return;
-    }
-    if (part != 0) return;
-    // the whole lane in one CTA, bucketed in global scratch
-    bucket_sort(seg, cnt, p.tmp + (size_t)lane * p.ecap, cnt, out, 0, m, s_hist, s_cur);
 }
 
 // Labels to the caller's layout (query-major, original vertex order): a CTA takes
@@ -364,11 +384,15 @@ cudaError_t iso_launch_emit(const isod::EmitParams& p, int K, int grid, cudaStre
     return cudaGetLastError();
 }
 
-cudaError_t iso_launch_sort_gather(const isod::GatherParams& p, int K, cudaStream_t s) {
+cudaError_t iso_launch_sort_gather(const isod::GatherParams& params, int K, cudaStream_t s) {
     const int smem = (kSortSmem + 2 * kMaxBuckets + 1) * 4;
     static std::atomic<unsigned long long> attr{0};
     if (cudaError_t e = iso_smem_attr_once(k_sort_gather, smem, attr)) return e;
-    k_sort_gather<<<K * kParts, kSortThreads, smem, s>>>(p);
+    GatherParams p = params;
+    // about 256 CTAs, which two per SM hold at once
+    p.part_bits = K >= 64 ? 2 : K >= 32 ? 3 : 4;
+    p.mult = p.m > (1 << kFineBits) ? (uint32_t)((1ull << (32 + kFineBits)) / (unsigned long long)p.m) : 0u;
+    k_sort_gather<<<K << p.part_bits, kSortThreads, smem, s>>>(p);
     return cudaGetLastError();
 }
 
