@@ -13,7 +13,8 @@ struct iso_graph_view {
     int device;  // CUDA device the graph was uploaded to
     int64_t m;
     const uint32_t *down_off, *up_off, *pair_off;
-    const int2 *down_arc, *up_arc, *pair_ids;
+    const int2 *down_arc, *pair_ids;
+    const int4* up_arc;
     const int32_t *pair_head, *pos, *level_off, *pair_owner;
     const uint2* core_arc;
     const uint32_t* level_arc;

@@ -151,7 +151,7 @@ struct iso_graph {
     uint32_t* down_off = nullptr;
     int2* down_arc = nullptr;
     uint32_t* up_off = nullptr;
-    int2* up_arc = nullptr;
+    int4* up_arc = nullptr;
     // emission: input arcs as vertex pairs by owner, owners in BFS order (emit_pairs.h)
     uint32_t* pair_off = nullptr;
     int32_t* pair_head = nullptr;
@@ -767,12 +767,25 @@ extern "C" int iso_upload_graph(const iso_ch* ch, const iso_alloc* alloc, void* 
         return ISO_E_NOMEM;
     }
     for (size_t i = 0; i <= n; ++i) off32[i] = (uint32_t)ch->up_off[i];
-    arcs.assign(ch->up_dst.size() + 2, make_int2(0, 0));
-    for (size_t i = 0; i < ch->up_dst.size(); ++i) arcs[i] = make_int2(ch->up_dst[i], ch->up_w[i]);
-    if ((rc = g->upload(&g->up_off, off32.data(), n + 1)) || (rc = g->upload(&g->up_arc, arcs.data(), arcs.size()))) {
-        free_all(); return rc;
+    try {
+        const size_t mu = ch->up_dst.size();
+        std::vector<int4> up(mu + kUpArcPad, make_int4(0, 0, -1, 1));
+        for (size_t v = 0; v < n; ++v)
+            for (size_t a = off32[v]; a < off32[v + 1]; ++a) {
+                const int32_t x = ch->up_dst[a];
+                up[a] = make_int4(x, ch->up_w[a], off32[x] < off32[x + 1] ? (int32_t)off32[x] : -1, a + 1 == off32[v + 1]);
+            }
+        if ((rc = g->upload(&g->up_off, off32.data(), n + 1)) || (rc = g->upload(&g->up_arc, up.data(), up.size()))) {
+            cudaStreamSynchronize(g->stream);  // no copy may outlive the host arrays
+            free_all();
+            return rc;
+        }
+        ISO_CK(cudaStreamSynchronize(g->stream));
+    } catch (const std::bad_alloc&) {
+        free_all();
+        iso::set_error("iso_upload_graph: out of host memory");
+        return ISO_E_NOMEM;
     }
-    ISO_CK(cudaStreamSynchronize(g->stream));
     try {
         EmitPairs ep;
         iso_make_emit_pairs(ch->n, ch->orig_off.data(), ch->orig_head.data(), ch->orig_id.data(), ch->bfs.data(), &ep);

@@ -27,6 +27,9 @@ constexpr uint32_t kInf = 0x7FFFFFFFu;
 constexpr int kCoreMaxVertices = 53248;
 constexpr int kCoreMaxLevels = 1023;
 
+// Entries past the upward arcs that a group of threads may read.
+constexpr int kUpArcPad = 16;
+
 // Device status word values (status[0]); the host maps them to ISO_E_*.
 enum : int {
     kStOk = 0,
@@ -41,7 +44,8 @@ enum : int { kStepWide = 0, kStepFused = 1 };
 
 struct UpParams {
     const uint32_t* up_off;   // [n+1]
-    const int2* up_arc;       // {dst, len}, dst a sweep position
+    const int4* up_arc;       // {dst, len, dst's first arc or -1 if it has none, last arc of its tail},
+                              // dst a sweep position; kUpArcPad more entries with the mark set
     const int32_t* pos;       // original id -> sweep position
     const int32_t* src;       // [K] original ids, -1 = idle lane
     const int32_t* tau;       // [K]
