@@ -544,8 +544,7 @@ def main():
     info = ws.sweep_info()
     # the sweep kernel that the options select (iso.h: sweep_kernel)
     chunked = any(opts.get(key) for key in ("threads_per_vertex", "ctas_per_sm", "fuse_width", "sweep_kernel",
-                                            "schedule_delay", "solo_width", "chunk_span", "restrict_sweep",
-                                            "fused_emission"))
+                                            "schedule_delay", "solo_width", "chunk_span", "fused_emission"))
     kern = ("k_core + " if info["core_levels"] else "") + (f"k_sweep_tma<{K}>" if chunked else f"k_tiles<{K}>")
     roof = {"bound": "hbm", "achieved": round(achieved, 1), "peak": peak, "unit": "GB/s",
             "frac": round(achieved / peak, 4), "traffic": traffic, "kernel": kern,

@@ -176,8 +176,8 @@ typedef struct {
     int32_t sweep_kernel;       /* 0 = auto: tiles swept out of shared memory, or the TMA-staged chunk
                                    schedule where another option asks for it (threads_per_vertex,
                                    ctas_per_sm, fuse_width, schedule_delay, solo_width, chunk_span,
-                                   debug_stage_*, restrict_sweep, fused_emission) or a vertex has too
-                                   many arcs for a tile; 1 = chunk schedule, 2 = plain loads */
+                                   debug_stage_*, fused_emission) or a vertex has too many arcs for a
+                                   tile; 1 = chunk schedule, 2 = plain loads */
     int32_t record_trace;       /* 1 = record the device time of every sweep step (iso_workspace_trace) */
     int32_t schedule_delay;     /* TMA-staged sweep: a chunk is scheduled at least this many positions
                                    after the chunks it depends on; 0 = auto (three times the CTA count) */
@@ -197,9 +197,9 @@ typedef struct {
                                    chunk in shared memory (0 = the buffer size, 3,072); chunks with
                                    more read their arcs from global memory */
     int32_t debug_stage_deps;   /* testing only: likewise for dependency-list entries (0 = 128) */
-    int32_t restrict_sweep;     /* TMA-staged sweep: 1 = skip the chunks that landmark lower bounds show
-                                   to be out of range for every query of the batch (Section 2's
-                                   restricted scan, Section 5's active cells); needs
+    int32_t restrict_sweep;     /* tile or TMA-staged sweep: 1 = skip the tiles or chunks that landmark
+                                   lower bounds show to be out of range for every query of the batch
+                                   (Section 2's restricted scan, Section 5's active cells); needs
                                    iso_graph_add_landmarks; 0 = sweep everything */
     int32_t fused_emission;     /* TMA-staged sweep: 1 = the sweep emits the isochrone edges itself
                                    (Section 5: each input arc is checked at its later-swept endpoint
@@ -294,7 +294,7 @@ typedef struct {
     int32_t reserved[4];
 } iso_sweep_info;
 int iso_workspace_sweep_info(const iso_workspace* ws, iso_sweep_info* out);
-/* Chunks the last collected batch skipped (restricted sweep; 0 otherwise). */
+/* Chunks (or tiles) the last collected batch skipped (restricted sweep; 0 otherwise). */
 int iso_workspace_skipped_chunks(const iso_workspace* ws, int64_t* out);
 /* Waits for the workspace's stream and frees its device buffers (into the
  * graph's allocator).  Free every workspace before the graph it was created

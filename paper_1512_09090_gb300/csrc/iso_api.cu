@@ -105,7 +105,7 @@ int core_limit_of(const iso_query_opts& o, int n) {
 bool wants_tiles(const iso_query_opts& o) {
     return o.sweep_kernel == 0 && o.threads_per_vertex == 0 && o.ctas_per_sm == 0 && o.fuse_width == 0 &&
            o.schedule_delay == 0 && o.solo_width == 0 && o.chunk_span == 0 && o.debug_stage_arcs == 0 &&
-           o.debug_stage_deps == 0 && o.restrict_sweep == 0 && o.fused_emission == 0;
+           o.debug_stage_deps == 0 && o.fused_emission == 0;
 }
 
 // Sweep kernel, threads per vertex, CTAs per SM and vertices per CTA batch that
@@ -384,6 +384,20 @@ int build_schedule(iso_workspace* ws) {
         in.max_chunk_deps = t.max_ext;
         in.arc_cap = t.lim.blob_bytes / 8;
         in.dep_cap = t.lim.rows;
+        ws->Q = t.count;
+        if (ws->restrict_sweep) {
+            // landmark bounds of every tile
+            const size_t words = std::max<size_t>((size_t)t.count * g->lm.count, 1);
+            ws->chunk_lo = (uint32_t*)ws->alloc(words * 4);
+            ws->chunk_hi = (uint32_t*)ws->alloc(words * 4);
+            ws->skip = (uint8_t*)ws->alloc(std::max<size_t>(t.count, 1));
+            if (!ws->chunk_lo || !ws->chunk_hi || !ws->skip) {
+                iso::set_error("workspace: device allocation failed");
+                return ISO_E_NOMEM;
+            }
+            ISO_CK(iso_launch_tile_bounds(t.dir, t.blob, t.count, g->n, g->lm.count, g->lm_fwd, g->lm_bwd, ws->chunk_lo,
+                                          ws->chunk_hi, ws->stream));
+        }
     } else if (ws->kernel == 1) {
         // TMA sweep: locality-ordered chunk schedule, cached on the graph
         const int delay = ws->sched_delay;

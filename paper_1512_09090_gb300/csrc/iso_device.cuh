@@ -106,8 +106,8 @@ struct SweepParams {
     // testing: stage at most this many arcs / dependency-list entries per chunk
     // (0 = the buffer sizes); larger chunks take the global-memory paths
     int stage_arc_cap, stage_pred_cap;
-    // restricted sweep: skip[q] != 0 = chunk at position q is out of range for
-    // every lane (k_skip); its rows are written kInf without gathers (nullable)
+    // restricted sweep: skip[q] != 0 = tile q, or the chunk at position q, is out of
+    // range for every lane (k_skip); its rows are written kInf without gathers (nullable)
     const uint8_t* skip;
     // fused emission (fused_emit != 0): the input arcs at their later-swept
     // endpoint v, emit_ent[emit_off[v] .. emit_off[v+1]) = {other endpoint, arc
@@ -242,3 +242,7 @@ cudaError_t iso_launch_sort_gather(const isod::GatherParams& p, int K, cudaStrea
 cudaError_t iso_launch_dist(const isod::DistParams& p, cudaStream_t s);
 cudaError_t iso_launch_range(const isod::RangeParams& p, int K, cudaStream_t s);
 cudaError_t iso_launch_skip(const isod::SkipParams& p, int grid, cudaStream_t s);
+// Landmark bounds of every tile of a plan: lo, hi [tiles * count] (k_skip.cu).
+cudaError_t iso_launch_tile_bounds(const uint2* dir, const uint4* blob, int tiles, int n, int count,
+                                   const uint32_t* lm_fwd, const uint32_t* lm_bwd, uint32_t* lo, uint32_t* hi,
+                                   cudaStream_t s);

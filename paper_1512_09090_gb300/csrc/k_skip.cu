@@ -1,4 +1,4 @@
-// Restricted sweep: the chunks of the schedule that are out of range for every
+// Restricted sweep: the tiles, or chunks of the schedule, that are out of range for every
 // lane of a batch (RPHAST's restricted scan, Section 2; isoPHAST's active
 // cells, Section 5, decide the same with precomputed cell distances).
 //
@@ -59,7 +59,41 @@ __global__ void __launch_bounds__(256) k_skip(SkipParams p) {
     if (threadIdx.x == 0 && s_count) atomicAdd(p.skipped, s_count);
 }
 
+// Per tile and landmark, the smallest d(L, v) and the largest d(v, L) over the
+// tile's own vertices (a warp per tile; once per workspace).
+__global__ void __launch_bounds__(256) k_tile_bounds(const uint2* dir, const uint4* blob, int tiles, int n, int count,
+                                                     const uint32_t* lm_fwd, const uint32_t* lm_bwd, uint32_t* lo,
+                                                     uint32_t* hi) {
+    const int lane = threadIdx.x & 31;
+    for (int q = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); q < tiles; q += (int)(gridDim.x * blockDim.x) >> 5) {
+        const uint32_t* rec = reinterpret_cast<const uint32_t*>(blob + __ldg(dir + q).x);
+        const int n_own = (int)__ldg(rec + 1);
+        const uint32_t* vert = rec + __ldg(rec + 3);
+        for (int l = 0; l < count; ++l) {
+            uint32_t a = kUnreach, b = 0;
+            for (int i = lane; i < n_own; i += 32) {
+                const uint32_t v = __ldg(vert + 2 * i) & ~kTileStore;
+                a = min(a, __ldg(lm_fwd + (size_t)l * n + v));
+                b = max(b, __ldg(lm_bwd + (size_t)l * n + v));
+            }
+            a = __reduce_min_sync(0xffffffffu, a);
+            b = __reduce_max_sync(0xffffffffu, b);
+            if (lane == 0) {
+                lo[(size_t)q * count + l] = a;
+                hi[(size_t)q * count + l] = b;
+            }
+        }
+    }
+}
+
 }  // namespace
+
+cudaError_t iso_launch_tile_bounds(const uint2* dir, const uint4* blob, int tiles, int n, int count,
+                                   const uint32_t* lm_fwd, const uint32_t* lm_bwd, uint32_t* lo, uint32_t* hi,
+                                   cudaStream_t s) {
+    if (tiles > 0) k_tile_bounds<<<1024, 256, 0, s>>>(dir, blob, tiles, n, count, lm_fwd, lm_bwd, lo, hi);
+    return cudaGetLastError();
+}
 
 cudaError_t iso_launch_skip(const isod::SkipParams& p, int grid, cudaStream_t s) {
     if (p.count <= 0 || p.count > kMaxLm || p.K > 64) return cudaErrorInvalidValue;
