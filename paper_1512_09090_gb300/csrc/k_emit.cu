@@ -105,7 +105,9 @@ __global__ void __launch_bounds__(kEmitThreads) k_emit(EmitParams p) {
                 if (x == 0) continue;
                 const int2 id = __ldg(p.ids + a);
                 const int each = id.y >= 0 ? 2 : 1;
-                for (int slot = atomicAdd(&s_n, each * __popcll(x)); x; x &= x - 1, slot += each) {
+                // (a full buffer's counter stands still, so it cannot wrap)
+                const bool full = *(volatile int*)&s_n >= kEmitBuffer;
+                for (int slot = full ? kEmitBuffer : atomicAdd(&s_n, each * __popcll(x)); x; x &= x - 1, slot += each) {
                     const int i = __ffsll((long long)x) - 1;
                     if (slot + each <= kEmitBuffer) {
                         const uint32_t to = (uint32_t)i << 24 | (uint32_t)atomicAdd(&s_cnt[i], each);

@@ -481,7 +481,8 @@ TileLimits iso_tile_limits(int K) {
     // ms of the whole sweep step: 64 lanes, rows 100 (5 CTAs) 2.58, 120 2.61, 156
     // (4 CTAs) 2.71, 80 (6 CTAs) 2.62; comp 16 2.58, 12 2.58, 8 2.64.  16 lanes: rows
     // 300 1.25, 400 1.27, 220 1.35.  8 lanes: rows 400 1.12, 600 1.14.  One lane: 24 KB
-    // records 0.83, 16 KB 0.89, 10 KB 0.90.
+    // records 0.83, 16 KB 0.89, 10 KB 0.90; comp 64 instead of 32 0.367 for 0.373 on 4M,
+    // 0.178 for 0.184 on 1M.
     TileLimits l{};
     switch (K) {
         case 64: l.rows = 100; l.blob_bytes = 6144; l.comp = 16; break;
@@ -489,7 +490,7 @@ TileLimits iso_tile_limits(int K) {
         case 16: l.rows = 300; l.blob_bytes = 10240; l.comp = 16; break;
         case 8: l.rows = 400; l.blob_bytes = 10240; l.comp = 24; break;
         case 4: l.rows = 1000; l.blob_bytes = 14336; l.comp = 32; break;
-        default: l.rows = 2500; l.blob_bytes = 24576; l.comp = 32; break;
+        default: l.rows = 2500; l.blob_bytes = 24576; l.comp = 64; break;
     }
     l.arcs = kTileArcs(K);
     l.width = kThreads / (K >= 8 ? K / 8 : 1);
