@@ -1306,7 +1306,8 @@ extern "C" int iso_query(iso_graph* g, int32_t k, const int32_t* sources, const 
         for (int i = 0; i < kb; ++i) offs[b + i + 1] = used + lo[i + 1];
         used += lo[kb];
     }
-    // (every batch has been waited for)
+    // (every batch has been waited for, and with it what was on the stream before)
+    if (k == 0) ISO_CK(cudaStreamSynchronize((cudaStream_t)stream));
     if (dev_off) {
         ISO_CK(cudaMemcpyAsync(out_offsets, offs.data(), offs.size() * 8, cudaMemcpyHostToDevice, (cudaStream_t)stream));
         ISO_CK(cudaStreamSynchronize((cudaStream_t)stream));
