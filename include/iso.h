@@ -192,7 +192,7 @@ typedef struct {
                                    they hold at most this many vertices in total, are swept for each
                                    lane by one CTA with the lane's labels in shared memory (Section 5's
                                    small top graph swept first); 0 = auto (the most that fit, 53,248;
-                                   20,000 above tiles), -1 = never */
+                                   10,000 or 20,000 above tiles), -1 = never */
     int32_t debug_stage_arcs;   /* testing only (TMA-staged sweep): stage at most this many arcs per
                                    chunk in shared memory (0 = the buffer size, 3,072); chunks with
                                    more read their arcs from global memory */

@@ -74,10 +74,12 @@ bool is_device_ptr(const void* p) {
 }
 
 constexpr int kMaxLanes = 64;
-// Largest per-lane core above the tiles, by default: the core's blocks cost one SM
-// more the wider they get, a tier of tiles about 15 us.  Sweep step on 18M, 64
-// lanes: 2.64 ms with 10,000 and with 20,000 vertices, 2.68 with 35,000.
-constexpr int kTileCore = 20000;
+// Largest per-lane core above the tiles, by default: a block of the core costs one
+// SM the more the wider it is, a tier of tiles about 15 us.  Sweep step in ms with
+// 5,000 / 10,000 / 20,000 / 35,000 vertices: one lane, 1M 0.168 / 0.164 / 0.179 / 0.219,
+// 4M 0.358 / 0.350 / 0.369 / 0.414; 64 lanes, 1M 0.312 / 0.293 / 0.303, 4M 0.762 /
+// 0.741 / 0.752; 16 lanes (and 32), 4M 0.526 / 0.504 / 0.493 / 0.518.
+int tile_core(int K) { return K == 16 || K == 32 ? 20000 : 10000; }
 // default size limit of the top levels that CTA 0 sweeps alone in the TMA
 // sweep (four vertices per consumer warp)
 constexpr int kSoloWidth = 124;
@@ -877,7 +879,7 @@ extern "C" int iso_workspace_create(iso_graph* g, int32_t lanes, const iso_query
     ws->core_limit = core_limit_of(o, g->n);
     ws->want_tiles = wants_tiles(o);
     if (ws->want_tiles) {
-        const int core = core_levels_of(g, o.core_vertices == 0 ? std::min(kTileCore, g->n) : ws->core_limit);
+        const int core = core_levels_of(g, o.core_vertices == 0 ? std::min(tile_core(ws->K), g->n) : ws->core_limit);
         const int per = iso_tiles_occupancy(ws->K, iso_tile_limits(ws->K));
         if (per > 0) ws->tiles = tile_plan(g, ws->K, g->h_level_off[core]);
         if (ws->tiles) {
