@@ -127,8 +127,12 @@ __global__ void __launch_bounds__(kEmitThreads) k_emit(EmitParams p) {
                 }
             }
         }
-        __syncthreads();
-        if (s_n > kEmitBuffer / 2) flush();  // (the same in every thread)
+        // The decision is the barrier's own result, so that it is one for the whole CTA: a
+        // thread that read s_n after the barrier could see what a faster warp has added in
+        // the next round.  (Each thread reads after its own appends, the last to append
+        // reads the final count, and the count only grows: some thread's answer is true
+        // iff the final count's is.)
+        if (__syncthreads_or(*(volatile int*)&s_n > kEmitBuffer / 2)) flush();
     }
     flush();
 }
