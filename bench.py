@@ -72,6 +72,11 @@ def lanes_class(k):
     return 64
 
 
+def sweep_name(info, K):
+    """The sweep kernel that a workspace with this sweep_info() runs at K lanes."""
+    return f"{('k_sweep', 'k_sweep_tma', 'k_tiles')[info['sweep']]}<{K}>"
+
+
 def max_over_ranks(x, dist=None, device="cpu"):
     """Largest x over all ranks (the job's time is its slowest rank's); x itself without a process group."""
     if dist is None:
@@ -540,12 +545,9 @@ def main():
     sw = statistics.mean(sweep_ms)
     peak, src = peaks()
     achieved = alg / (sw / 1e3) / 1e9
-    traffic = sweep_traffic(args.workload, opts)
     info = ws.sweep_info()
-    # the sweep kernel that the options select (iso.h: sweep_kernel)
-    chunked = any(opts.get(key) for key in ("threads_per_vertex", "ctas_per_sm", "fuse_width", "sweep_kernel",
-                                            "schedule_delay", "solo_width", "chunk_span", "fused_emission"))
-    kern = ("k_core + " if info["core_levels"] else "") + (f"k_sweep_tma<{K}>" if chunked else f"k_tiles<{K}>")
+    kern = ("k_core + " if info["core_levels"] else "") + sweep_name(info, K)
+    traffic = sweep_traffic(args.workload, opts) if sweep_name(info, K).startswith("k_tiles") else None
     roof = {"bound": "hbm", "achieved": round(achieved, 1), "peak": peak, "unit": "GB/s",
             "frac": round(achieved / peak, 4), "traffic": traffic, "kernel": kern,
             "alg_bytes_per_launch": alg, "alg_bytes_design": alg_design,

@@ -291,7 +291,9 @@ typedef struct {
     int32_t chunks_over_arc_cap; /* chunks whose arcs are read from global memory */
     int32_t chunks_over_dep_cap; /* chunks whose dependency list is checked in global memory */
     int32_t arc_cap, dep_cap;    /* staging limits in force */
-    int32_t reserved[4];
+    int32_t sweep;               /* the sweep that runs: 0 plain, 1 chunk schedule, 2 tiles (options that
+                                    leave the choice to the library get 1 where there are no tiles) */
+    int32_t reserved[3];
 } iso_sweep_info;
 int iso_workspace_sweep_info(const iso_workspace* ws, iso_sweep_info* out);
 /* Chunks (or tiles) the last collected batch skipped (restricted sweep; 0 otherwise). */

@@ -384,6 +384,7 @@ int build_schedule(iso_workspace* ws) {
     if (ws->tiles) {
         const TileDevice& t = *ws->tiles;
         iso_sweep_info& in = ws->info;
+        in.sweep = 2;
         in.levels = g->L;
         in.core_levels = in.solo_levels = in.sync_levels = ws->core_levels;
         in.core_vertices = ws->core_n;
@@ -444,6 +445,7 @@ int build_schedule(iso_workspace* ws) {
         ws->Q = sc->Q;
         {
             iso_sweep_info& in = ws->info;
+            in.sweep = 1;
             in.levels = g->L;
             in.core_levels = core;
             in.core_vertices = ws->core_n;
