@@ -110,6 +110,13 @@ bool wants_tiles(const iso_query_opts& o) {
            o.debug_stage_deps == 0 && o.fused_emission == 0;
 }
 
+// Largest per-lane core above the tiles that options o ask for on K lanes (core_vertices
+// = 0: the library's, not the chunk schedule's), or -1 where they ask for another sweep.
+int tile_core_limit_of(const iso_query_opts& o, int K, int n) {
+    if (!wants_tiles(o)) return -1;
+    return o.core_vertices == 0 ? std::min(tile_core(K), n) : core_limit_of(o, n);
+}
+
 // Sweep kernel, threads per vertex, CTAs per SM and vertices per CTA batch that
 // options o select for K lanes.  Returns false if the combination is unsupported.
 bool sweep_shape(int K, const iso_query_opts& o, int* kernel, int* tpv, int* occ, int* vpb) {
@@ -241,7 +248,7 @@ struct iso_workspace {
     int Q = 0;
     unsigned long long* upmask = nullptr;  // [n] TMA sweep: lanes with upward labels
     uint32_t* core_out = nullptr;  // [K * core_n] TMA sweep: the per-lane core's labels, lane-major
-    bool want_tiles = false;       // the options leave the sweep to the library
+    int tile_core_limit = -1;      // largest core above tiles (-1: the options name another sweep)
     std::shared_ptr<TileDevice> tiles;  // tile sweep (null: chunk schedule or plain sweep)
     int vpb = 0;
     int2* pairs = nullptr;
@@ -879,9 +886,9 @@ extern "C" int iso_workspace_create(iso_graph* g, int32_t lanes, const iso_query
     ws->solo_width = o.solo_width < 0 ? 0 : (o.solo_width > 0 ? o.solo_width : kSoloWidth);
     ws->chunk_span = o.chunk_span;
     ws->core_limit = core_limit_of(o, g->n);
-    ws->want_tiles = wants_tiles(o);
-    if (ws->want_tiles) {
-        const int core = core_levels_of(g, o.core_vertices == 0 ? std::min(tile_core(ws->K), g->n) : ws->core_limit);
+    ws->tile_core_limit = tile_core_limit_of(o, ws->K, g->n);
+    if (ws->tile_core_limit >= 0) {
+        const int core = core_levels_of(g, ws->tile_core_limit);
         const int per = iso_tiles_occupancy(ws->K, iso_tile_limits(ws->K));
         if (per > 0) ws->tiles = tile_plan(g, ws->K, g->h_level_off[core]);
         if (ws->tiles) {
@@ -1253,9 +1260,9 @@ bool same_config(const iso_workspace* ws, const iso_query_opts& o) {
     const int per_sm = o.ctas_per_sm ? std::min<int>(o.ctas_per_sm, occ) : occ;
     const int fuse = o.fuse_width == 0 ? vpb : (o.fuse_width < 0 ? 0 : o.fuse_width);
     const long long timeout = o.barrier_timeout_ns ? o.barrier_timeout_ns : 2000000000LL;
-    const bool tiles = wants_tiles(o);  // (then the grid is the tile sweep's, the same for all such options)
-    return ws->kernel == kernel && ws->tpv == tpv && ws->want_tiles == tiles &&
-           (tiles || ws->grid == ws->g->num_sms * per_sm) &&
+    const int tiles = tile_core_limit_of(o, ws->K, ws->g->n);  // (where there are, the grid is the tile sweep's)
+    return ws->kernel == kernel && ws->tpv == tpv && ws->tile_core_limit == tiles &&
+           (tiles >= 0 || ws->grid == ws->g->num_sms * per_sm) &&
            ws->fuse_width == fuse && ws->use_graph == (o.use_cuda_graph != 0) && ws->timeout_ns == timeout &&
            ws->bar_extra == o.debug_barrier_extra && ws->record_trace == (o.record_trace != 0 && kernel == 1) &&
            ws->sched_delay == (o.schedule_delay > 0 ? o.schedule_delay : 3 * ws->g->num_sms * per_sm) &&
