@@ -193,6 +193,7 @@ struct iso_graph {
     };
     std::vector<CachedSchedule> schedules;
     std::vector<std::shared_ptr<TileDevice>> plans;  // tile plans in use or used lately (kMaxPlans idle ones at most)
+    std::vector<std::pair<int, int>> no_plan;        // {lanes, core vertices} for which there is none
     std::mutex plan_mu;
     std::mutex mu;
     iso_workspace* query_ws[7] = {};
@@ -325,11 +326,14 @@ int core_levels_of(const iso_graph* g, int limit) {
 
 // The tile plan for K lanes below a core of core_n vertices (built once per
 // graph and kept while a workspace uses it), or null where there is none: a
-// vertex with too many sources, or no memory for it.
+// vertex with too many sources (found once per graph and remembered: building a
+// plan takes seconds on 18M vertices, refused or not), or no memory for it.
 std::shared_ptr<TileDevice> tile_plan(iso_graph* g, int K, int core_n) {
     std::lock_guard<std::mutex> lock(g->plan_mu);
     for (auto& t : g->plans)
         if (t->K == K && t->core_n == core_n) return t;
+    for (const auto& none : g->no_plan)
+        if (none.first == K && none.second == core_n) return nullptr;
     auto t = std::make_shared<TileDevice>();
     t->A = g->A;
     t->stream = g->stream;
@@ -338,9 +342,10 @@ std::shared_ptr<TileDevice> tile_plan(iso_graph* g, int K, int core_n) {
     t->lim = iso_tile_limits(K);
     try {
         TilePlan plan;
-        if (iso_make_tiles(g->n, g->L, g->h_level_off.data(), g->h_down_off.data(), g->h_down_src.data(),
-                           g->h_down_len.data(), g->h_bfs.data(), core_n, t->lim, &plan) != 0)
-            return nullptr;
+        const int rc = iso_make_tiles(g->n, g->L, g->h_level_off.data(), g->h_down_off.data(), g->h_down_src.data(),
+                                      g->h_down_len.data(), g->h_bfs.data(), core_n, t->lim, &plan);
+        if (rc == -1) g->no_plan.emplace_back(K, core_n);
+        if (rc != 0) return nullptr;
         t->tiers = plan.tiers;
         t->count = plan.tier_off.back();
         t->max_arcs = plan.max_arcs;
@@ -887,16 +892,6 @@ extern "C" int iso_workspace_create(iso_graph* g, int32_t lanes, const iso_query
     ws->chunk_span = o.chunk_span;
     ws->core_limit = core_limit_of(o, g->n);
     ws->tile_core_limit = tile_core_limit_of(o, ws->K, g->n);
-    if (ws->tile_core_limit >= 0) {
-        const int core = core_levels_of(g, ws->tile_core_limit);
-        const int per = iso_tiles_occupancy(ws->K, iso_tile_limits(ws->K));
-        if (per > 0) ws->tiles = tile_plan(g, ws->K, g->h_level_off[core]);
-        if (ws->tiles) {
-            ws->core_levels = core;
-            ws->core_n = g->h_level_off[core];
-            ws->grid = g->num_sms * per;
-        }
-    }
     ws->stage_arc_cap = o.debug_stage_arcs;
     ws->stage_pred_cap = o.debug_stage_deps;
     ws->restrict_sweep = o.restrict_sweep != 0;
@@ -909,6 +904,16 @@ extern "C" int iso_workspace_create(iso_graph* g, int32_t lanes, const iso_query
         iso::set_error("iso_workspace_create: restrict_sweep needs landmarks on the graph (iso_graph_add_landmarks) "
                        "and the TMA-staged sweep");
         return ISO_E_INVAL;
+    }
+    if (ws->tile_core_limit >= 0) {  // (the options are good: a plan may take long to build)
+        const int core = core_levels_of(g, ws->tile_core_limit);
+        const int per = iso_tiles_occupancy(ws->K, iso_tile_limits(ws->K));
+        if (per > 0) ws->tiles = tile_plan(g, ws->K, g->h_level_off[core]);
+        if (ws->tiles) {
+            ws->core_levels = core;
+            ws->core_n = g->h_level_off[core];
+            ws->grid = g->num_sms * per;
+        }
     }
     ws->use_graph = opts ? opts->use_cuda_graph != 0 : false;
     if (opts && opts->barrier_timeout_ns) ws->timeout_ns = opts->barrier_timeout_ns;

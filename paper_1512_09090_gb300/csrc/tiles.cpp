@@ -79,7 +79,7 @@ struct Job {
     int32_t lo, hi;  // components by_order[lo .. hi)
     std::vector<uint32_t> dir, blob;
     int max_arcs = 0, max_ext = 0;
-    bool ok = true;
+    bool ok = true, no_memory = false;
 };
 
 }  // namespace
@@ -374,10 +374,16 @@ int iso_make_tiles(int n, int L, const int32_t* level_off, const uint32_t* down_
             }
         } catch (const std::bad_alloc&) {
             job.ok = false;
+            job.no_memory = true;
         }
         if (!job.ok) failed.store(true);
     }
-    if (failed.load()) return -1;
+    if (failed.load()) {
+        // (a job that found a vertex too large says so whatever became of the others)
+        for (const Job& j : jobs)
+            if (!j.ok && !j.no_memory) return -1;
+        return -2;
+    }
     // jobs are in sweep order (highest tier first): join their records
     out->tier_off.assign((size_t)tiers + 1, 0);
     size_t words = 0, tiles = 0;

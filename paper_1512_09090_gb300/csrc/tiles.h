@@ -42,8 +42,8 @@ struct TilePlan {
 
 // Builds the plan for sweep positions [core_n, n).  down_off/src/len: incoming
 // downward arcs by sweep position (arcs of length 0x7FFFFFFF never lower a
-// label and are left out); bfs: spatial key of each position.  Returns 0, or
-// -1 if some vertex cannot be placed within the limits (the caller then uses
-// the chunk schedule).
+// label and are left out); bfs: spatial key of each position.  Returns 0;
+// -1 if some vertex cannot be placed within the limits, whenever it is tried, or -2
+// if memory ran out (the caller then uses the chunk schedule).
 int iso_make_tiles(int n, int L, const int32_t* level_off, const uint32_t* down_off, const int32_t* down_src,
                    const int32_t* down_len, const int32_t* bfs, int core_n, const TileLimits& lim, TilePlan* out);
