@@ -54,7 +54,9 @@ struct Allocator {
         bytes = (bytes + 255) & ~(size_t)255;
         if (custom) return cb.alloc(cb.ctx, bytes, s);
         void* p = nullptr;
-        return cudaMalloc(&p, bytes) == cudaSuccess ? p : nullptr;
+        if (cudaMalloc(&p, bytes) == cudaSuccess) return p;
+        cudaGetLastError();  // (reported by the null; a launch after it must not see it)
+        return nullptr;
     }
     void put(void* p, cudaStream_t s) {
         if (!p) return;
@@ -199,9 +201,26 @@ struct iso_graph {
     iso_workspace* query_ws[7] = {};
     std::vector<void*> owned;
 
+    // Frees the tile plans that no workspace uses (the caller holds plan_mu); false: there were none.
+    bool drop_idle_plans() {
+        const size_t had = plans.size();
+        plans.erase(std::remove_if(plans.begin(), plans.end(), [](auto& t) { return t.use_count() == 1; }), plans.end());
+        return plans.size() < had;
+    }
+    // Device memory; where it is short, idle tile plans make room.
+    void* get(size_t bytes, cudaStream_t s) {
+        void* p = A.get(bytes, s);
+        if (p) return p;
+        {
+            std::lock_guard<std::mutex> lock(plan_mu);
+            if (!drop_idle_plans()) return nullptr;
+        }
+        return A.get(bytes, s);
+    }
+
     template <class T>
     int upload(T** dst, const T* src, size_t count) {
-        *dst = (T*)A.get(count * sizeof(T), stream);
+        *dst = (T*)get(count * sizeof(T), stream);
         if (!*dst) { iso::set_error("iso_upload_graph: device allocation of %zu bytes failed", count * sizeof(T)); return ISO_E_NOMEM; }
         owned.push_back(*dst);
         if (count) ISO_CK(cudaMemcpyAsync(*dst, src, count * sizeof(T), cudaMemcpyHostToDevice, stream));
@@ -292,7 +311,7 @@ struct iso_workspace {
     size_t ctl_words() const { return 8 + 2 * (size_t)K; }
 
     void* alloc(size_t bytes) {
-        void* p = g->A.get(bytes, stream);
+        void* p = g->get(bytes, stream);
         if (p) owned.push_back(p);
         return p;
     }
@@ -334,13 +353,13 @@ std::shared_ptr<TileDevice> tile_plan(iso_graph* g, int K, int core_n) {
         if (t->K == K && t->core_n == core_n) return t;
     for (const auto& none : g->no_plan)
         if (none.first == K && none.second == core_n) return nullptr;
-    auto t = std::make_shared<TileDevice>();
-    t->A = g->A;
-    t->stream = g->stream;
-    t->K = K;
-    t->core_n = core_n;
-    t->lim = iso_tile_limits(K);
     try {
+        auto t = std::make_shared<TileDevice>();
+        t->A = g->A;
+        t->stream = g->stream;
+        t->K = K;
+        t->core_n = core_n;
+        t->lim = iso_tile_limits(K);
         TilePlan plan;
         const int rc = iso_make_tiles(g->n, g->L, g->h_level_off.data(), g->h_down_off.data(), g->h_down_src.data(),
                                       g->h_down_len.data(), g->h_bfs.data(), core_n, t->lim, &plan);
@@ -353,6 +372,7 @@ std::shared_ptr<TileDevice> tile_plan(iso_graph* g, int K, int core_n) {
         auto put = [&](auto** dst, const auto& v) {
             const size_t bytes = v.size() * sizeof(v[0]);
             *(void**)dst = g->A.get(bytes, g->stream);
+            if (!*dst && g->drop_idle_plans()) *(void**)dst = g->A.get(bytes, g->stream);
             return *dst && (bytes == 0 || cudaMemcpyAsync(*dst, v.data(), bytes, cudaMemcpyHostToDevice, g->stream) ==
                                               cudaSuccess);
         };
@@ -362,14 +382,14 @@ std::shared_ptr<TileDevice> tile_plan(iso_graph* g, int K, int core_n) {
             cudaGetLastError();
             return nullptr;
         }
+        for (size_t i = 0; i < g->plans.size() && g->plans.size() >= kMaxPlans;)
+            if (g->plans[i].use_count() == 1) g->plans.erase(g->plans.begin() + i);
+            else ++i;
+        g->plans.push_back(t);
+        return t;
     } catch (const std::bad_alloc&) {
         return nullptr;
     }
-    for (size_t i = 0; i < g->plans.size() && g->plans.size() >= kMaxPlans;)
-        if (g->plans[i].use_count() == 1) g->plans.erase(g->plans.begin() + i);
-        else ++i;
-    g->plans.push_back(t);
-    return t;
 }
 
 int build_schedule(iso_workspace* ws) {
@@ -861,11 +881,11 @@ extern "C" void iso_free_graph(iso_graph* g) {
     delete g;
 }
 
-extern "C" int iso_workspace_create(iso_graph* g, int32_t lanes, const iso_query_opts* opts, void* stream,
-                                    iso_workspace** out) {
-    iso::clear_error();
-    if (!g || !out) { iso::set_error("iso_workspace_create: NULL argument"); return ISO_E_INVAL; }
-    *out = nullptr;
+namespace {
+// A workspace with the sweep that the options select, or (tiles = false) the chunk
+// schedule in place of tiles.
+int create_workspace(iso_graph* g, int32_t lanes, const iso_query_opts* opts, void* stream, bool tiles,
+                     iso_workspace** out) {
     if (lanes < 1 || lanes > kMaxLanes) { iso::set_error("iso_workspace_create: lanes must be in 1..64"); return ISO_E_INVAL; }
     int rc = check_opts(opts);
     if (rc) return rc;
@@ -905,7 +925,7 @@ extern "C" int iso_workspace_create(iso_graph* g, int32_t lanes, const iso_query
                        "and the TMA-staged sweep");
         return ISO_E_INVAL;
     }
-    if (ws->tile_core_limit >= 0) {  // (the options are good: a plan may take long to build)
+    if (tiles && ws->tile_core_limit >= 0) {  // (the options are good: a plan may take long to build)
         const int core = core_levels_of(g, ws->tile_core_limit);
         const int per = iso_tiles_occupancy(ws->K, iso_tile_limits(ws->K));
         if (per > 0) ws->tiles = tile_plan(g, ws->K, g->h_level_off[core]);
@@ -925,6 +945,9 @@ extern "C" int iso_workspace_create(iso_graph* g, int32_t lanes, const iso_query
         if (ws->h_ctl) cudaFreeHost(ws->h_ctl);
         if (ws->h_out) cudaFreeHost(ws->h_out);
         ws->h_io = ws->h_ctl = ws->h_out = nullptr;
+        for (auto& e : ws->ev)
+            if (e) cudaEventDestroy(e);
+        if (ws->ev_swept) cudaEventDestroy(ws->ev_swept);
         return code;
     };
     const size_t n = (size_t)g->n, K = (size_t)ws->K;
@@ -981,6 +1004,22 @@ extern "C" int iso_workspace_create(iso_graph* g, int32_t lanes, const iso_query
     if (ws->restrict_sweep) ++g->restricted_ws;
     *out = ws.release();
     return ISO_OK;
+}
+}  // namespace
+
+extern "C" int iso_workspace_create(iso_graph* g, int32_t lanes, const iso_query_opts* opts, void* stream,
+                                    iso_workspace** out) {
+    iso::clear_error();
+    if (!g || !out) { iso::set_error("iso_workspace_create: NULL argument"); return ISO_E_INVAL; }
+    *out = nullptr;
+    int rc = create_workspace(g, lanes, opts, stream, true, out);
+    // A tile plan takes more memory than a chunk schedule (1.03 GB at 64 lanes on 18M
+    // vertices): without room for both a plan and the rest, the chunk schedule it is.
+    if (rc == ISO_E_NOMEM && wants_tiles(opts ? *opts : iso_query_opts{})) {
+        iso::clear_error();
+        rc = create_workspace(g, lanes, opts, stream, false, out);
+    }
+    return rc;
 }
 
 extern "C" void iso_free_workspace(iso_workspace* ws) {
