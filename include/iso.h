@@ -293,7 +293,9 @@ typedef struct {
     int32_t arc_cap, dep_cap;    /* staging limits in force */
     int32_t sweep;               /* the sweep that runs: 0 plain, 1 chunk schedule, 2 tiles (options that
                                     leave the choice to the library get 1 where there are no tiles) */
-    int32_t reserved[3];
+    int32_t plan_kib;            /* device memory (KiB) of the tile plan made along with this workspace, which
+                                    later workspaces of its kind share (0: no plan, or it was there) */
+    int32_t reserved[2];
 } iso_sweep_info;
 int iso_workspace_sweep_info(const iso_workspace* ws, iso_sweep_info* out);
 /* Chunks (or tiles) the last collected batch skipped (restricted sweep; 0 otherwise). */

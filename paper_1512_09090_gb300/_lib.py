@@ -76,7 +76,7 @@ class SweepInfo(ctypes.Structure):
     _fields_ = [(k, ctypes.c_int32) for k in ("levels", "core_levels", "core_vertices", "solo_levels",
                                               "sync_levels", "chunks", "max_chunk_arcs", "max_chunk_deps",
                                               "chunks_over_arc_cap", "chunks_over_dep_cap", "arc_cap",
-                                              "dep_cap", "sweep")] + [("reserved", ctypes.c_int32 * 3)]
+                                              "dep_cap", "sweep", "plan_kib")] + [("reserved", ctypes.c_int32 * 2)]
 
     def as_dict(self):
         return {k: getattr(self, k) for k, _ in self._fields_ if k != "reserved"}

@@ -144,6 +144,7 @@ struct TileDevice {
     cudaStream_t stream = nullptr;
     int K = 0, core_n = 0, tiers = 0, count = 0, max_arcs = 0, max_ext = 0;
     TileLimits lim{};
+    size_t bytes = 0;  // device memory
     int32_t* off = nullptr;
     uint2* dir = nullptr;
     uint4* blob = nullptr;
@@ -347,7 +348,9 @@ int core_levels_of(const iso_graph* g, int limit) {
 // graph and kept while a workspace uses it), or null where there is none: a
 // vertex with too many sources (found once per graph and remembered: building a
 // plan takes seconds on 18M vertices, refused or not), or no memory for it.
-std::shared_ptr<TileDevice> tile_plan(iso_graph* g, int K, int core_n) {
+// *made_kib: its size if it was built by this call, else 0.
+std::shared_ptr<TileDevice> tile_plan(iso_graph* g, int K, int core_n, int32_t* made_kib) {
+    *made_kib = 0;
     std::lock_guard<std::mutex> lock(g->plan_mu);
     for (auto& t : g->plans)
         if (t->K == K && t->core_n == core_n) return t;
@@ -373,6 +376,7 @@ std::shared_ptr<TileDevice> tile_plan(iso_graph* g, int K, int core_n) {
             const size_t bytes = v.size() * sizeof(v[0]);
             *(void**)dst = g->A.get(bytes, g->stream);
             if (!*dst && g->drop_idle_plans()) *(void**)dst = g->A.get(bytes, g->stream);
+            t->bytes += bytes;
             return *dst && (bytes == 0 || cudaMemcpyAsync(*dst, v.data(), bytes, cudaMemcpyHostToDevice, g->stream) ==
                                               cudaSuccess);
         };
@@ -386,6 +390,7 @@ std::shared_ptr<TileDevice> tile_plan(iso_graph* g, int K, int core_n) {
             if (g->plans[i].use_count() == 1) g->plans.erase(g->plans.begin() + i);
             else ++i;
         g->plans.push_back(t);
+        *made_kib = (int32_t)(t->bytes >> 10);
         return t;
     } catch (const std::bad_alloc&) {
         return nullptr;
@@ -928,7 +933,7 @@ int create_workspace(iso_graph* g, int32_t lanes, const iso_query_opts* opts, vo
     if (tiles && ws->tile_core_limit >= 0) {  // (the options are good: a plan may take long to build)
         const int core = core_levels_of(g, ws->tile_core_limit);
         const int per = iso_tiles_occupancy(ws->K, iso_tile_limits(ws->K));
-        if (per > 0) ws->tiles = tile_plan(g, ws->K, g->h_level_off[core]);
+        if (per > 0) ws->tiles = tile_plan(g, ws->K, g->h_level_off[core], &ws->info.plan_kib);
         if (ws->tiles) {
             ws->core_levels = core;
             ws->core_n = g->h_level_off[core];

@@ -14,7 +14,8 @@ Admission by device memory: the pool starts with `workspaces` workspaces and
 grows by one (up to max_workspaces) whenever requests are left waiting behind
 busy workspaces and the device still has room for another one -- free memory,
 read when the growth is considered, must cover a workspace's measured size
-within `memory_fraction` of what is free.  A workspace is warmed (one batch,
+(without the tile plan, which all of them share) within `memory_fraction` of
+what is free.  A workspace is warmed (one batch,
 which also captures its CUDA graph) before it takes requests.
 
 Host work per batch is kept out of per-request Python: requests are taken from
@@ -119,7 +120,9 @@ class IsoServer:
         first = self._new_workspace()
         torch.cuda.synchronize()
         free1, _ = torch.cuda.mem_get_info()
-        self.bytes_per_workspace = max(free0 - free1, 1)
+        # (a tile plan made with the first workspace serves the later ones too)
+        plan = first.sweep_info()["plan_kib"] << 10 if hasattr(first, "sweep_info") else 0
+        self.bytes_per_workspace = max(free0 - free1 - plan, 1)
         self.workspaces = [first]
         for _ in range(max(1, workspaces or 1) - 1):
             self.workspaces.append(self._new_workspace())

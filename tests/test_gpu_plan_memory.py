@@ -78,3 +78,19 @@ def test_idle_plans_make_room(monkeypatch):
     ws.free()
     dg.free()
     assert mem.live == 0
+
+
+def test_a_plan_is_reported_by_the_workspace_that_made_it(monkeypatch):
+    g = synth.grid_road_graph(250, 200, seed=9)
+    dg, mem = upload(P.iso_build_ch(g.n, g.tail, g.head, g.weight), monkeypatch)
+    took = []
+    for k in (16, 16, 64):
+        before = mem.live
+        ws = P.Workspace(dg, k)
+        took.append((ws.sweep_info()["plan_kib"], mem.live - before))
+        ws.free()
+    assert took[0][0] > 0 and took[1][0] == 0 and took[2][0] > 0
+    # (allocations are rounded up to 256 bytes each)
+    assert 0 <= took[0][1] - took[1][1] - (took[0][0] << 10) < 2048
+    P.Workspace(dg, 64, sweep_kernel=1).free()
+    dg.free()
