@@ -5,6 +5,8 @@
 #include <cstdint>
 #include <vector>
 
+#include "host_arrays.h"
+
 // What one tile may hold (the kernel's shared-memory layout, per lane class).
 struct TileLimits {
     int rows;        // label rows in shared memory: sources from outside + own vertices read inside
@@ -35,7 +37,7 @@ struct TilePlan {
     int tiers = 0;
     std::vector<int32_t> tier_off;   // [tiers + 1] first tile of each tier, in sweep order
     std::vector<uint32_t> dir;       // per tile {record start / 16 bytes, record bytes}
-    std::vector<uint32_t> blob;      // the records
+    Raw<uint32_t> blob;              // the records
     std::vector<int32_t> level_tier; // [L] last tier with vertices of each level block (-1: core)
     int max_arcs = 0, max_ext = 0;   // extremes over the tiles
 };
