@@ -4,12 +4,14 @@
 #include <cstdint>
 #include <vector>
 
+#include "host_arrays.h"
+
 // Pairs of vertices joined by input arcs, listed at the endpoint of lower BFS
 // rank (the owner), in the order of the owners' ranks.
 struct EmitPairs {
     std::vector<uint32_t> off;       // [n + 1] first pair of each owner, by BFS rank
-    std::vector<int32_t> head;       // the other endpoint's sweep position
-    std::vector<int32_t> ids;        // per pair {arc id, second arc id or -1}
+    Raw<int32_t> head;               // the other endpoint's sweep position
+    Raw<int32_t> ids;                // per pair {arc id, second arc id or -1}
 };
 
 // orig_off/head/id: input arcs grouped by tail, by sweep position; bfs: BFS rank of
