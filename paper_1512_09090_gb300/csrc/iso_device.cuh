@@ -28,7 +28,7 @@ constexpr int kCoreMaxVertices = 53248;
 constexpr int kCoreMaxLevels = 1023;
 
 // Entries past the upward arcs that a group of threads may read.
-constexpr int kUpArcPad = 16;
+constexpr int kUpArcPad = 32;
 
 // Device status word values (status[0]); the host maps them to ISO_E_*.
 enum : int {
