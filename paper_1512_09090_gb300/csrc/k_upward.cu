@@ -30,7 +30,7 @@ using namespace isod;
 constexpr int kThreads = 1024;
 constexpr int kSmemSlots = 16384;  // power of two; at most half of them occupied
 
-constexpr int kSmemFrontier = 3072;  // frontier entries in shared memory
+constexpr int kSmemFrontier = 3072;  // frontier entries in shared memory (the rest in global memory)
 constexpr int kGroup = 16;           // threads per frontier vertex where a warp each is not enough
 constexpr int kOverflow = 1 << 28;   // frontier size that says the table overflowed
 
@@ -38,10 +38,11 @@ struct Table {
     int32_t* key;        // vertex or -1
     uint32_t* dist;      // label
     uint32_t* queued[2]; // bitmaps: slot is in the frontier of an even / odd round
-    uint2* fr[2];        // frontiers {slot, first arc}
+    uint2* fr[2];        // frontiers {slot, first arc}: entries below fcap ...
+    uint2* more[2];      // ... and those from fcap on, minus fcap
     uint32_t mask;       // slots - 1
-    int limit;           // maximum occupied slots
-    int fcap;            // frontier capacity
+    int limit;           // maximum occupied slots, and frontier entries
+    int fcap;
 };
 
 // key, dist, two bitmaps, two frontiers
@@ -75,6 +76,7 @@ __device__ __forceinline__ Table carve(uint32_t* base, uint32_t slots, uint32_t 
     t.queued[1] = t.queued[0] + slots / 32;
     t.fr[0] = (uint2*)(t.queued[1] + slots / 32);
     t.fr[1] = t.fr[0] + fcap;
+    t.more[0] = t.more[1] = nullptr;
     t.mask = slots - 1;
     t.limit = (int)(slots / 2);
     t.fcap = (int)fcap;
@@ -105,42 +107,53 @@ __device__ bool search(const Table& t, const UpParams& p, int32_t s, uint32_t ta
     for (int r = 0;; ++r) {
         nfr = s_nfr[r % 3];  // (nobody changes it in this round)
         if (nfr == 0 || nfr >= kOverflow) break;
-        const uint2* cur = t.fr[r & 1];
-        uint2* nxt = t.fr[(r + 1) & 1];
         if (threadIdx.x == 0) s_nfr[(r + 2) % 3] = 0;  // last read in round r - 1
         const int gs = nfr > kThreads / 32 ? kGroup : 32;  // threads per frontier vertex
         const int gl = threadIdx.x & (gs - 1);
         const unsigned peers = gs == 32 ? 0xFFFFFFFFu : 0xFFFFu << (threadIdx.x & 16);  // the group's of the warp
-        for (int f = threadIdx.x / gs; f < nfr; f += kThreads / gs) {
-            const uint2 me = cur[f];
-            const int su = (int)me.x;
-            // the vertex leaves its queue; an improvement in this round re-queues it in the other one
-            if (gl == 0) atomicAnd(&t.queued[r & 1][su >> 5], ~(1u << (su & 31)));
-            const uint32_t du = *((volatile uint32_t*)&t.dist[su]);
-            const int4* at = p.up_arc + (me.y + gl);
-            int4 next = __ldg(at);  // (the array goes on for a group past its end)
-            for (;;) {
-                const int4 arc = next;
-                const unsigned last = __ballot_sync(peers, arc.w != 0) & peers;
-                if (!last) next = __ldg(at += gs);  // (a long list: on its way meanwhile)
-                const bool mine = !last || (threadIdx.x & 31) <= __ffs(last) - 1;
-                const uint32_t nd = du + (uint32_t)arc.y;
-                if (mine && nd <= tau) {
-                    const int sx = find_or_insert(t, arc.x, &s_used);
-                    if (sx < 0) {
-                        atomicMax(&s_nfr[(r + 1) % 3], kOverflow);
-                    } else if (nd < atomicMin(&t.dist[sx], nd) && arc.z != -1) {
-                        const uint32_t bit = 1u << (sx & 31);
-                        if (!(atomicOr(&t.queued[(r + 1) & 1][sx >> 5], bit) & bit)) {
-                            const int i = atomicAdd(&s_nfr[(r + 1) % 3], 1);
-                            if (i < t.fcap) nxt[i] = make_uint2((uint32_t)sx, (uint32_t)arc.z);
-                            else atomicMax(&s_nfr[(r + 1) % 3], kOverflow);
+        uint2* cur = t.fr[r & 1];
+        uint2* nxt = t.fr[(r + 1) & 1];
+        for (int f0 = 0;;) {
+            const int n = min(nfr - f0, t.fcap);
+            for (int f = threadIdx.x / gs; f < n; f += kThreads / gs) {
+                const uint2 me = cur[f];
+                const int su = (int)me.x;
+                // the vertex leaves its queue; an improvement in this round re-queues it in the other one
+                if (gl == 0) atomicAnd(&t.queued[r & 1][su >> 5], ~(1u << (su & 31)));
+                const uint32_t du = *((volatile uint32_t*)&t.dist[su]);
+                const int4* at = p.up_arc + (me.y + gl);
+                int4 next = __ldg(at);  // (the array goes on for a group past its end)
+                for (;;) {
+                    const int4 arc = next;
+                    const unsigned last = __ballot_sync(peers, arc.w != 0) & peers;
+                    if (!last) next = __ldg(at += gs);  // (a long list: on its way meanwhile)
+                    const bool mine = !last || (threadIdx.x & 31) <= __ffs(last) - 1;
+                    const uint32_t nd = du + (uint32_t)arc.y;
+                    if (mine && nd <= tau) {
+                        const int sx = find_or_insert(t, arc.x, &s_used);
+                        if (sx < 0) {
+                            atomicMax(&s_nfr[(r + 1) % 3], kOverflow);
+                        } else if (nd < atomicMin(&t.dist[sx], nd) && arc.z != -1) {
+                            const uint32_t bit = 1u << (sx & 31);
+                            if (!(atomicOr(&t.queued[(r + 1) & 1][sx >> 5], bit) & bit)) {
+                                const int i = atomicAdd(&s_nfr[(r + 1) % 3], 1);
+                                const uint2 x = make_uint2((uint32_t)sx, (uint32_t)arc.z);
+                                if (i < t.fcap) nxt[i] = x;
+                                else if (i < t.limit) t.more[(r + 1) & 1][i - t.fcap] = x;
+                                else atomicMax(&s_nfr[(r + 1) % 3], kOverflow);
+                            }
                         }
                     }
+                    if (last) break;
+                    __syncwarp(peers);
                 }
-                if (last) break;
-                __syncwarp(peers);
             }
+            // (rare: the part of the frontier that the shared one did not hold takes its place)
+            f0 += t.fcap;
+            if (f0 >= nfr) break;
+            __syncthreads();
+            for (int f = threadIdx.x; f < min(nfr - f0, t.fcap); f += kThreads) cur[f] = t.more[r & 1][f0 - t.fcap + f];
+            __syncthreads();
         }
         __syncthreads();
     }
@@ -192,11 +205,20 @@ __global__ void __launch_bounds__(kThreads) k_upward(UpParams p) {
         return;
     }
     const int32_t s = p.pos[src];
-    const bool small_cap = !p.direct && p.cap < kSmemSlots / 2;   // pairs must hold every label
-    if (!small_cap && search(carve(smem, kSmemSlots, kSmemFrontier), p, s, (uint32_t)tau, lane)) return;
+    uint32_t* base = p.gtab + (size_t)lane * iso_upward_table_words_of(p.gcap);
+    // A table in shared memory holds all its vertices as one frontier too: what goes past
+    // the shared part lies where the global table would be.  (Source of 7,000 arcs to
+    // vertices with arcs of their own: 575 us when such a search was redone in global
+    // memory for its frontier, now 189.)  Not where the pairs cannot hold every label.
+    const bool fits = (p.direct || p.cap >= kSmemSlots / 2) && p.gcap >= kSmemSlots / 2;
+    if (fits) {
+        Table t = carve(smem, kSmemSlots, kSmemFrontier);
+        t.more[0] = (uint2*)base;
+        t.more[1] = t.more[0] + (kSmemSlots / 2 - kSmemFrontier);
+        if (search(t, p, s, (uint32_t)tau, lane)) return;
+    }
     // Too large for shared memory: the same search on this lane's global table.
     __syncthreads();
-    uint32_t* base = p.gtab + (size_t)lane * iso_upward_table_words_of(p.gcap);
     if (!search(carve(base, (uint32_t)p.gcap, (uint32_t)p.gcap / 2), p, s, (uint32_t)tau, lane)) {
         if (threadIdx.x == 0) { p.cnt[lane] = 0; atomicCAS(p.status, kStOk, kStUpOverflow); }
     }

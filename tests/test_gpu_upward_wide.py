@@ -30,6 +30,16 @@ def depot(yards):
     return yards + 1 + GATES, tail, head, (np.arange(tail.size) * 7919 % 97 + 1).astype(np.int32)
 
 
+def hubs(yards):
+    """The same with three roads from each gate to other gates, which keeps the gates above
+    the yards: every yard is in the frontier of the second round."""
+    n, tail, head, weight = depot(yards)
+    g = yards + 1 + np.arange(GATES, dtype=np.int32)
+    more = 3 * GATES
+    return (n, np.concatenate([tail, g, g, g]), np.concatenate([head, np.roll(g, -1), np.roll(g, -2), np.roll(g, -3)]),
+            np.concatenate([weight, (np.arange(more) * 31 % 89 + 1).astype(np.int32)]))
+
+
 def run(dg, graph, k, yards, **opts):
     srcs = (np.arange(k) % 3 * (yards // 2)).astype(np.int32)  # the depot and two yards
     taus = (200 - np.arange(k)).astype(np.int32)
@@ -44,6 +54,24 @@ def test_wide_searches(yards):
     dg = P.iso_upload_graph(P.iso_build_ch(*graph))
     for k, opts in ((1, {}), (5, dict(core_vertices=-1)), (64, dict(use_cuda_graph=1)), (4, dict(sweep_kernel=2))):
         run(dg, graph, k, yards, **opts)
+    dg.free()
+
+
+# a frontier of shared memory's 3,072 entries, and one, two and three times as many to
+# come from global memory; the last ones about the table's limit
+@pytest.mark.parametrize("yards", [33, 3071, 3072, 3073, 3100, 6143, 6144, 6145, 7000, 8180, 8183, 8184, 8190, 8200])
+def test_wide_frontiers(yards):
+    graph = hubs(yards)
+    dg = P.iso_upload_graph(P.iso_build_ch(*graph))
+    for k, opts in ((1, {}), (64, dict(use_cuda_graph=1)), (4, dict(sweep_kernel=2))):
+        run(dg, graph, k, yards, **opts)
+    # the allocation-free call (tables of 8,192 vertices; 93% of the yards are within 90)
+    srcs, taus = np.zeros(3, np.int32), np.array([90, 40, 0], np.int32)
+    off, arcs, _ = P.iso_query(dg, srcs, taus)
+    d_off = torch.zeros(4, dtype=torch.int64, device="cuda")
+    d_arcs = torch.zeros(int(off[-1]), dtype=torch.int32, device="cuda")
+    P._lib.iso_query_noalloc(dg, torch.from_numpy(srcs).cuda(), torch.from_numpy(taus).cuda(), d_off, d_arcs)
+    assert np.array_equal(d_off.cpu().numpy(), off) and np.array_equal(d_arcs.cpu().numpy(), arcs)
     dg.free()
 
 
