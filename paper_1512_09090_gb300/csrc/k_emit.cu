@@ -178,8 +178,11 @@ __global__ void __launch_bounds__(kEmitThreads, 8) k_emit(EmitParams p) {
 // twice: to count the ids of every part and of its own buckets, and, after a scan,
 // to scatter its own ids into their buckets in shared memory.  Small buckets
 // (about four ids) are then sorted by one thread each (insertion sort), larger
-// ones by the whole CTA (every id's place is the number of smaller ids in its
-// bucket).  The parts' sorted lists are consecutive pieces of the lane's.  CTA 0
+// ones by a warp or the whole CTA (every id's place is the number of smaller ids
+// in its bucket; a thread alone took up to 40 us for 64 ids: one list of 1,006 ids
+// in two runs of neighbours among 2M, 45 us, now 16).  The ranking loops' registers
+// (48) leave one CTA per SM: held to 32, crowded lists took up to 2.7 times as long
+// and spread ones no less.  The parts' sorted lists are consecutive pieces of the lane's.  CTA 0
 // also writes the offsets.  A lane one of whose parts would not fit shared memory
 // is sorted by its part-0 CTA alone with the list in global memory.
 //
@@ -188,7 +191,8 @@ __global__ void __launch_bounds__(kEmitThreads, 8) k_emit(EmitParams p) {
 // a ten-step scan, now 0.057; one query (15,000 ids) 0.061 with four CTAs, now 0.024.
 constexpr int kFineBits = 14;
 constexpr int kMaxBuckets = 4096;
-constexpr int kSmallBucket = 64;
+constexpr int kSmallBucket = 16;
+constexpr int kWarpBucket = 128;
 constexpr int kMaxBigBuckets = 256;  // big buckets listed for the whole-CTA ranking
 constexpr int kMaxParts = 16;
 
@@ -229,8 +233,8 @@ __global__ void __launch_bounds__(kSortThreads) k_sort_gather(GatherParams p) {
     // buckets per part: about four ids each if all of the list lies in one part, which it
     // does where ids follow the map.  Made for lists spread over the parts, buckets of such
     // ids held up to sixteen times as many, and ranking them takes the square: 3,000
-    // neighbouring ids of 2M in 64 lists 223 us, now 84; one list on 1M vertices with ids in
-    // the order of the map, limit 3,600, 60, now 25; spread ids 16.4 and 12.3 as before.
+    // neighbouring ids of 2M in 64 lists 223 us, now 49; one list on 1M vertices with ids in
+    // the order of the map, limit 3,600, 60, now 17; spread ids 16 and 12 as before.
     int lg = 0;
     while (lg < kFineBits - p.part_bits && (1 << lg) < kMaxBuckets && (4 << lg) < cnt) ++lg;
     int pbits = p.part_bits;
@@ -309,11 +313,15 @@ __global__ void __launch_bounds__(kSortThreads) k_sort_gather(GatherParams p) {
         }
     }
     __syncthreads();
+    bool more = false;  // a bucket that is not small
     for (int bb = tid; bb < nb; bb += kSortThreads) {
         const int blo = s_hist[bb], bhi = s_hist[bb + 1];
         if (bhi - blo > kSmallBucket) {
-            const int q = atomicAdd(&s_nbig, 1);
-            if (q < kMaxBigBuckets) s_big[q] = bb;
+            more = true;
+            if (bhi - blo > kWarpBucket) {
+                const int q = atomicAdd(&s_nbig, 1);
+                if (q < kMaxBigBuckets) s_big[q] = bb;
+            }
             continue;
         }
         for (int i = blo + 1; i < bhi; ++i) {
@@ -323,21 +331,33 @@ __global__ void __launch_bounds__(kSortThreads) k_sort_gather(GatherParams p) {
             B[j + 1] = x;
         }
     }
+    more = __syncthreads_or(more);
+    // sorted buckets go out together (coalesced); the others' places are written over
+    for (int i = tid; i < my; i += kSortThreads) out[i] = B[i];
+    if (!more) return;
     __syncthreads();
-    // sorted buckets go out together (coalesced); big ones are ranked by the whole
-    // CTA, from the list of them or, if it overflowed, bucket by bucket
-    const int nbig = s_nbig;
-    if (nbig == 0) {
-        for (int i = tid; i < my; i += kSortThreads) out[i] = B[i];
-        return;
+    // buckets of middling size are ranked by a warp each, of the 32 its threads look at
+    // (neighbours, which are crowded together, go to different warps)
+    for (int b0 = 0; b0 < nb; b0 += kSortThreads) {
+        const int bb = b0 + wl * (kSortThreads / 32) + warp;
+        const int blo = bb < nb ? s_hist[bb] : 0, c = bb < nb ? s_hist[bb + 1] - blo : 0;
+        for (unsigned mid = __ballot_sync(0xffffffffu, c > kSmallBucket && c <= kWarpBucket); mid; mid &= mid - 1) {
+            const int lo = __shfl_sync(0xffffffffu, blo, __ffs(mid) - 1);
+            const int hi = lo + __shfl_sync(0xffffffffu, c, __ffs(mid) - 1);
+            for (int i = lo + wl; i < hi; i += 32) {
+                const int32_t x = B[i];
+                int r = 0;
+                for (int j = lo; j < hi; ++j) r += B[j] < x;
+                out[lo + r] = x;
+            }
+        }
     }
-    for (int bb = tid; bb < nb; bb += kSortThreads)
-        if (s_hist[bb + 1] - s_hist[bb] <= kSmallBucket)
-            for (int i = s_hist[bb]; i < s_hist[bb + 1]; ++i) out[i] = B[i];
+    // big ones by the whole CTA, from the list of them or, if it overflowed, bucket by bucket
+    const int nbig = s_nbig;
     for (int t = 0; t < (nbig <= kMaxBigBuckets ? nbig : nb); ++t) {
         const int bb = nbig <= kMaxBigBuckets ? s_big[t] : t;
         const int blo = s_hist[bb], bhi = s_hist[bb + 1];
-        if (bhi - blo <= kSmallBucket) continue;
+        if (bhi - blo <= kWarpBucket) continue;
         for (int i = blo + tid; i < bhi; i += kSortThreads) {
             const int32_t x = B[i];
             int r = 0;
