@@ -78,9 +78,15 @@ bool is_device_ptr(const void* p) {
 constexpr int kMaxLanes = 64;
 // Largest per-lane core above the tiles, by default: a block of the core costs one
 // SM the more the wider it is, a tier of tiles about 15 us.  Sweep step in ms with
-// 5,000 / 10,000 / 20,000 / 35,000 vertices: one lane, 1M 0.168 / 0.164 / 0.179 / 0.219,
-// 4M 0.358 / 0.350 / 0.369 / 0.414; 64 lanes, 1M 0.312 / 0.293 / 0.303, 4M 0.762 /
-// 0.741 / 0.752; 16 lanes (and 32), 4M 0.526 / 0.504 / 0.493 / 0.518.
+// 5,000 / 10,000 / 20,000 / 35,000 vertices:
+//   lanes  1M                       4M                       18M
+//   64     .315 / .299 / .306 / .338  .765 / .743 / .750 / .779  2.457 / 2.434 / 2.448 / 2.485
+//   32     .279 / .259 / .262 / .288  .606 / .582 / .586 / .610  1.681 / 1.658 / 1.657 / 1.689
+//   16     .264 / .240 / .242 / .271  .520 / .499 / .493 / .521  1.271 / 1.230 / 1.237 / 1.262
+//   8      .230 / .211 / .219 / .250  .469 / .457 / .457 / .487  1.122 / 1.104 / 1.106 / 1.146
+//   4      .191 / .182 / .197 / .227  .387 / .379 / .397 / .435   .909 /  .899 /  .915 /  .964
+//   1      .170 / .166 / .184 / .215  .352 / .353 / .369 / .411   .797 /  .788 /  .805 /  .859
+// (at 16 and 32 lanes 10,000 and 20,000 are within 1.3% of each other either way).
 int tile_core(int K) { return K == 16 || K == 32 ? 20000 : 10000; }
 // default size limit of the top levels that CTA 0 sweeps alone in the TMA
 // sweep (four vertices per consumer warp)
@@ -104,8 +110,8 @@ int core_limit_of(const iso_query_opts& o, int n) {
 
 // The sweep goes tile by tile (k_tiles) unless an option asks for one of the other
 // kernels or shapes the chunk schedule: the tiles were faster on every graph and
-// lane class measured (18M: 2.45 against 3.72 ms at 64 lanes, 0.83 against 1.27 at
-// one; 1M: 0.31 against 0.48 and 0.21 against 0.35).
+// lane class measured (18M: 2.44 against 3.72 ms at 64 lanes, 0.79 against 1.27 at
+// one; 1M: 0.30 against 0.48 and 0.17 against 0.35).
 bool wants_tiles(const iso_query_opts& o) {
     return o.sweep_kernel == 0 && o.threads_per_vertex == 0 && o.ctas_per_sm == 0 && o.fuse_width == 0 &&
            o.schedule_delay == 0 && o.solo_width == 0 && o.chunk_span == 0 && o.debug_stage_arcs == 0 &&

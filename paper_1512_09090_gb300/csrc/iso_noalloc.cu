@@ -46,7 +46,7 @@ constexpr int kMaxUpward = kUpCap / 2;
 constexpr int kMaxArcs = ISO_NOALLOC_MAX_ARCS;       // isochrone edges per query
 // The top of the hierarchy, at most this many vertices, is swept per lane by one CTA
 // (k_core): its blocks cost 1 us each there and 7 us each as grid-wide steps (1M
-// vertices: 112 of 130 blocks; four queries 1.04 ms without a core, now 0.59).
+// vertices: 97 of 130 blocks; four queries 1.04 ms without a core, now 0.58).
 constexpr int kCore = 20000;
 static_assert(kCore <= kCoreMaxVertices && kCore <= kMaxArcs, "the core's labels take the sort's scratch");
 

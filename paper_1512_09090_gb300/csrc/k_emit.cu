@@ -31,7 +31,7 @@ constexpr int kSortSmem = 16384;  // ids bucketed in shared memory (64 KB): two 
 // counter each: one atomicAdd per warp, query and round (half a million of them on
 // 64 counters in two cache lines) kept the kernel at 0.32 ms however many warps it
 // had.  18M vertices, 64 queries (1.2M edges): 0.52 ms arc by arc with those
-// atomics, now 0.23 (0.35 GB to move); one query 0.34, now 0.16.
+// atomics, now 0.22 (0.35 GB to move); one query 0.34, now 0.15.
 template <int K>
 __global__ void __launch_bounds__(kEmitThreads, 8) k_emit(EmitParams p) {
     using MaskT = typename MaskOf<K>::T;
@@ -188,7 +188,7 @@ __global__ void __launch_bounds__(kEmitThreads, 8) k_emit(EmitParams p) {
 //
 // Bound by latency (5 MB of ids): two passes over the longest list.  18M vertices,
 // 64 queries (1.2M ids): 0.20 ms with three passes, two 64-bit divisions an id and
-// a ten-step scan, now 0.057; one query (15,000 ids) 0.061 with four CTAs, now 0.024.
+// a ten-step scan, now 0.058; one query (15,000 ids) 0.061 with four CTAs, now 0.028.
 constexpr int kFineBits = 14;
 constexpr int kMaxBuckets = 4096;
 constexpr int kSmallBucket = 16;

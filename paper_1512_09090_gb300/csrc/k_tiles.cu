@@ -18,16 +18,17 @@
 // Restricted sweeps: a tile that landmark bounds show out of range for every query
 // (k_skip.cu) fetches no rows and sweeps nothing.  Tiles are compact, so their bounds
 // skip more than those of the chunk schedule's strips: one query with limit 3,600 on
-// 4M vertices skips 9,493 of 9,767 tiles; the call took 0.87 ms over chunks, 0.48 now.
-// Tiles of one tier are independent; a grid barrier separates the tiers (20 on
-// 18M vertices).  All waits are bounded (status word).
+// 4M vertices skips 9,339 to 9,632 of 9,902 tiles (three sources); the call took 0.87 ms
+// over chunks, 0.44 now.
+// Tiles of one tier are independent; a grid barrier separates the tiers (18M
+// vertices: 27 at 64 lanes, 17 at one).  All waits are bounded (status word).
 //
 // Bound: latency.  A tile of 50 vertices takes a CTA about 5 us, of which the rows
 // from outside are a third and five phases the rest (a phase: a serial chain of
 // shared-memory reads per four arcs of its largest vertex).  The sweep step (with
-// k_core) on 18M vertices, one GB300: 64 lanes 2.45 ms (chunk schedule 3.72), 32
-// lanes 1.66 (2.39), 16 lanes 1.25 (2.03), 8 lanes 1.12 (1.93), 4 lanes 0.92 (1.34),
-// one lane 0.83 (1.27); 1M: 64 lanes 0.31 (0.48), one lane 0.21 (0.35).
+// k_core, default core) on 18M vertices, one GB300: 64 lanes 2.44 ms (chunk schedule
+// 3.72), 32 lanes 1.66 (2.39), 16 lanes 1.24 (2.03), 8 lanes 1.10 (1.93), 4 lanes 0.90
+// (1.34), one lane 0.79 (1.27); 1M: 64 lanes 0.30 (0.48), one lane 0.17 (0.35).
 #include "sweep_device.cuh"
 
 namespace {
@@ -101,7 +102,7 @@ __device__ __forceinline__ uint32_t ld_relaxed_u32(const uint32_t* a) {
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 constexpr int kThreads = 128;
-constexpr int kCtasPerSm = 5;     // what the limits below leave room for
+constexpr int kCtasPerSm = 5;     // most that the limits below leave room for
 
 constexpr int kUpRows = 16;       // rows for upward labels (more flagged vertices read theirs in place)
 constexpr int kInPlace = kUpRows + 1;
@@ -116,8 +117,8 @@ struct TileSmem {
 // round r is over at (r + 1) * CTAs.  Bounded like grid_sync, and like it false, the
 // same on every thread, once the kernel has failed.  Against grid_sync's arrival
 // counter and generation word, one atomic round trip less for each of the barriers:
-// the sweep step takes 0.184 ms instead of 0.193 on 1M vertices (one lane), 1.23
-// instead of 1.25 on 18M (16 lanes).
+// the sweep step took 0.184 ms instead of 0.193 on 1M vertices (one lane, a core of
+// 19,000), 1.23 instead of 1.25 on 18M (16 lanes).
 __device__ bool tier_sync(const SweepParams& p, uint32_t& round) {
     __shared__ int s_ok;
     __syncthreads();
@@ -475,10 +476,11 @@ cudaError_t launch(const SweepParams& p, int grid, cudaStream_t s) {
 }  // namespace
 
 TileLimits iso_tile_limits(int K) {
-    // Five CTAs per SM (about 43 KB each): a tile costs mostly latency (rows from
+    // CTAs per SM: five at 64, 16 and 8 lanes, four at 32 and 4, three at one (by shared
+    // memory, 37 to 64 KB each, and at 8 lanes by registers).  A tile costs mostly latency (rows from
     // outside 1.4 us, 0.5 us a phase), so tiles in flight count for more than large
-    // tiles, except with one lane, where a tile's own work is small.  18M vertices,
-    // ms of the whole sweep step: 64 lanes, rows 100 (5 CTAs) 2.58, 120 2.61, 156
+    // tiles, except with one lane, where a tile's own work is small.  18M vertices with a
+    // core of 19,000, ms of the whole sweep step: 64 lanes, rows 100 (5 CTAs) 2.58, 120 2.61, 156
     // (4 CTAs) 2.71, 80 (6 CTAs) 2.62; comp 16 2.58, 12 2.58, 8 2.64.  16 lanes: rows
     // 300 1.25, 400 1.27, 220 1.35.  8 lanes: rows 400 1.12, 600 1.14.  One lane: 24 KB
     // records 0.83, 16 KB 0.89, 10 KB 0.90; comp 64 instead of 32 0.367 for 0.373 on 4M,

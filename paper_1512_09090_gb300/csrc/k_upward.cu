@@ -19,8 +19,9 @@
 // Bound by latency: a chain of rounds (about 90 on 18M vertices).  So a round has
 // one load from global memory in its chain -- an arc record says where its head's
 // own arcs start, and the last arc of a vertex is marked -- and one CTA barrier.
-// With the arc range looked up first, three barriers a round and a warp per vertex:
-// 0.19 ms for one search on 18M vertices, now 0.18; 64 searches 0.47, now 0.36.
+// With the arc range looked up first and three barriers a round: 0.19 ms for one search
+// on 18M vertices, 64 searches 0.47; without, 0.18 and 0.36.  (Five other batches, half
+// a warp per vertex throughout: 0.223 and 0.319, now 0.206 and 0.300.)
 #include "iso_device.cuh"
 
 namespace {
